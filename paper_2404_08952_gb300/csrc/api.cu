@@ -55,10 +55,18 @@ void init_paths()
     std::memset(g_batch, 0, sizeof g_batch);
     register_indicator(g_ind);
     register_batch(g_batch);
-    register_paths_d2s(g_paths);
-    register_paths_d2e(g_paths);
-    register_paths_d3s(g_paths);
-    register_paths_d3e(g_paths);
+    register_paths_d2s_f64(g_paths);
+    register_paths_d2s_f32(g_paths);
+    register_paths_d2s_bf16(g_paths);
+    register_paths_d2e_f64(g_paths);
+    register_paths_d2e_f32(g_paths);
+    register_paths_d2e_bf16(g_paths);
+    register_paths_d3s_f64(g_paths);
+    register_paths_d3s_f32(g_paths);
+    register_paths_d3s_bf16(g_paths);
+    register_paths_d3e_f64(g_paths);
+    register_paths_d3e_f32(g_paths);
+    register_paths_d3e_bf16(g_paths);
 }
 
 size_t al256(size_t b) { return (b + 255) & ~(size_t)255; }
@@ -353,12 +361,31 @@ std::string scheme_key(const dolinc_mesh *m, const dolinc_scheme *s)
     return k.str();
 }
 
+constexpr int64_t kTreeCells = 16384;
+
 Tune tune_for(const dolinc_mesh *m, const dolinc_scheme *s)
 {
     auto it = m->tuned.find(scheme_key(m, s));
     if (it != m->tuned.end()) return it->second;
-    Tune t;                                       // heuristic: one lane per face slot
-    t.diff_lpc = t.stage_lpc = m->max_faces <= 4 ? 4 : 8;
+    Tune t;
+    const int lanes = m->max_faces <= 4 ? 4 : 8;
+    t.diff_lpc = t.stage_lpc = lanes;             // one lane per face slot
+    if (s->precision == DOLINC_FP64) {
+        t.diff_lpc = pair_scheme(s) ? 2 : 1;
+        t.diff_block = 64;
+        t.stage_lpc = -2;
+        t.stage_block = 64;
+    } else if (m->max_faces <= lanes && m->h.n_cells >= kTreeCells) {
+        t.diff_lpc = 1;
+        t.diff_block = 64;
+        t.tree = lanes;
+        // WENO5's weights amplify the rounding of its fused products, which the compiler
+        // chooses per kernel: its stage keeps the lane kernel and that kernel's bits
+        if (s->limiter != DOLINC_LIMIT_WENO5_ALL && s->limiter != DOLINC_LIMIT_WENO5_FLAGGED) {
+            t.stage_lpc = -2;
+            t.stage_block = 64;
+        }
+    }
     return t;
 }
 

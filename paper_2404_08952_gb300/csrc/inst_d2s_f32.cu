@@ -1,0 +1,8 @@
+// Instantiations of the stage paths for dim = 2, 1 variable(s), F32.
+#include "launch.cuh"
+
+namespace dol {
+
+void register_paths_d2s_f32(PathFns *t) { register_paths<2, 1, PREC_F32>(t); }
+
+}  // namespace dol

@@ -1,0 +1,8 @@
+// Instantiations of the stage paths for dim = 3, 5 variable(s), BF16.
+#include "launch.cuh"
+
+namespace dol {
+
+void register_paths_d3e_bf16(PathFns *t) { register_paths<3, 5, PREC_BF16>(t); }
+
+}  // namespace dol

@@ -144,6 +144,12 @@ __global__ void __launch_bounds__(256) k_pack(int n, const double *__restrict__ 
     store_rec<typename PrecT<PREC>::T0, NV, rec_stride(NV, (int)sizeof(typename PrecT<PREC>::T0))>(o0, c, v);
 }
 
+// Correctly rounded products and sums that the compiler may not fuse: the increment
+// arithmetic is then the same in every stage kernel, whatever each one inlines.
+__device__ __forceinline__ float mul_rn(float x, float y) { return __fmul_rn(x, y); }
+__device__ __forceinline__ float add_rn(float x, float y) { return __fadd_rn(x, y); }
+__device__ __forceinline__ double add_rn(double x, double y) { return __dadd_rn(x, y); }
+
 // ------------------------------------------------------------------ differential pass
 // LPC lanes per cell: lane l gathers slots l, l+LPC, ... (lane 0 adds the cell's own
 // term), the group sums by recursive halving and each lane stores its slice of the
@@ -284,6 +290,138 @@ __device__ __forceinline__ void diff_cells(const DevMesh &mesh, const void *__re
     }
 }
 
+// The pass of TREE lanes per cell, by one thread per cell: the same sums in the same
+// order, so the same bits.  Lane l of a TREE-lane group holds A_l = slot l's term (lane
+// 0 the own term plus slot 0's) and group_reduce_scatter adds
+//   TREE 4:  (A0 + A2) + (A1 + A3)
+//   TREE 8:  ((A0 + A4) + (A2 + A6)) + ((A1 + A5) + (A3 + A7)),
+// a lane without a slot adding zero.  Cells have at most TREE slots (checked by the
+// launcher).  A pair of lanes is loaded at a time (all of them when the records are
+// small), so that their gathers overlap.
+// Why one thread: TREE lanes hold TREE accumulators, exchange them by shuffles and leave
+// lanes idle (5.3 of 8 on hexes and prisms); the pass then waits on issue slots and
+// shuffles instead of on memory.
+template <int DIM, int NV, int M, int PREC, int TREE>
+__device__ __forceinline__ void diff_cells_tree(const DevMesh &mesh, const void *__restrict__ in_v,
+                                                void *__restrict__ out_v, int c, int t, int nt, long long c0,
+                                                unsigned char *smo)
+{
+    using R = typename PrecT<PREC>::R;
+    using TI = typename OrdT<PREC, M - 1>::T;
+    using TO = typename OrdT<PREC, M>::T;
+    constexpr int CI = ncoef(DIM, M - 1), CO = ncoef(DIM, M);
+    constexpr int SI = ord_stride<DIM, NV, M - 1, PREC>(), SO = ord_stride<DIM, NV, M, PREC>();
+    const TI *in = static_cast<const TI *>(in_v);
+    TO *out = static_cast<TO *>(out_v);
+    const bool valid = c < mesh.n_cells;
+    R acc[NV * CO];
+#pragma unroll
+    for (int i = 0; i < NV * CO; ++i) acc[i] = (R)0;
+    if (valid) {
+        int s0, s1;
+        slot_range(mesh, c, s0, s1);
+        const int ns = s1 - s0;
+        // slots in the order the tree adds them, two at a time: (0, H), (2, H + 2), (1, ..)
+        constexpr int H = TREE / 2, NP = TREE / 2;
+        constexpr bool ALL = NV * CI <= 10;          // small records: every gather before the first sum
+        constexpr int NB = ALL ? NP : 1;
+        R kx[NB][2], ky[NB][2], kz[NB][2], x[NB][2][NV * CI];
+        // TREE 4: pairs (0,2) (1,3); TREE 8: (0,4) (2,6) (1,5) (3,7)
+        auto first = [](int p) { return TREE == 4 ? p : (p == 1 ? 2 : p == 2 ? 1 : p); };
+        auto load_pair = [&](int b, int p) {
+            int nb[2];
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int l = first(p) + h * H;
+                R kb = (R)0;
+                if (l < ns) ld4<R>(Geo<R>::slotk(mesh) + 4ll * (s0 + l), kx[b][h], ky[b][h], kz[b][h], kb);
+                nb[h] = Geo<R>::nb_of(kb);
+            }
+#pragma unroll
+            for (int h = 0; h < 2; ++h)
+                if (first(p) + h * H < ns) load_rec<TI, NV * CI, SI, R>(in, nb[h], x[b][h]);
+        };
+        if constexpr (ALL) {
+#pragma unroll
+            for (int p = 0; p < NP; ++p) load_pair(p, p);
+        } else {
+            load_pair(0, 0);
+        }
+        {
+            R own[NV * CI], wx, wy, wz, iv;
+            ld4<R>(Geo<R>::cellk(mesh) + 4ll * c, wx, wy, wz, iv);
+            load_rec<TI, NV * CI, SI, R>(in, c, own);
+            poly_mul_acc<DIM, NV, M, R>(acc, own, wx, wy, wz);
+        }
+        // one variable's term of slot h of batch b, from zero (the lane's own accumulator)
+        auto term = [&](int b, int h, int v, R *q) {
+#pragma unroll
+            for (int i = 0; i < CO; ++i) q[i] = (R)0;
+            poly_mul_acc<DIM, 1, M, R>(q, x[b][h] + v * CI, kx[b][h], ky[b][h], kz[b][h]);
+        };
+        R tmp[TREE == 8 ? NV * CO : 1];
+#pragma unroll
+        for (int p = 0; p < NP; ++p) {
+            const int b = ALL ? p : 0;
+            if (!ALL && p > 0) load_pair(0, p);
+            const bool on0 = first(p) < ns, on1 = first(p) + H < ns;
+#pragma unroll
+            for (int v = 0; v < NV; ++v) {
+                R q0[CO], q1[CO];
+                if (p == 0) {
+                    // lane 0: own term, then slot 0, in one accumulator; lane H added to it
+                    if (on0) poly_mul_acc<DIM, 1, M, R>(acc + v * CO, x[b][0] + v * CI, kx[b][0], ky[b][0], kz[b][0]);
+                    if (on1) {
+                        term(b, 1, v, q1);
+#pragma unroll
+                        for (int i = 0; i < CO; ++i) acc[v * CO + i] = add_rn(acc[v * CO + i], q1[i]);
+                    }
+                } else if (on0) {
+                    term(b, 0, v, q0);
+                    if (on1) {
+                        term(b, 1, v, q1);
+#pragma unroll
+                        for (int i = 0; i < CO; ++i) q0[i] = add_rn(q0[i], q1[i]);
+                    }
+                    if (TREE == 8 && p == 2) {
+#pragma unroll
+                        for (int i = 0; i < CO; ++i) tmp[v * CO + i] = q0[i];
+                    } else if (TREE == 8 && p == 3) {
+#pragma unroll
+                        for (int i = 0; i < CO; ++i) tmp[v * CO + i] = add_rn(tmp[v * CO + i], q0[i]);
+                    } else {
+#pragma unroll
+                        for (int i = 0; i < CO; ++i) acc[v * CO + i] = add_rn(acc[v * CO + i], q0[i]);
+                    }
+                }
+                if (TREE == 8 && p == 3) {
+#pragma unroll
+                    for (int i = 0; i < CO; ++i) acc[v * CO + i] = add_rn(acc[v * CO + i], tmp[v * CO + i]);
+                }
+            }
+        }
+    }
+    constexpr unsigned RBO = SO * (unsigned)sizeof(TO);
+    if constexpr (RBO % 16 == 0) {
+        if (valid) store_rec_smem<TO, NV * CO, SO, R>(smo, t, acc);
+        fence_proxy_async_smem();
+        __syncthreads();
+        if (t == 0 && c0 < mesh.n_cells) {
+            const unsigned n = (unsigned)min((long long)nt, (long long)mesh.n_cells - c0);
+            bulk_s2g_wait(out + c0 * SO, smo, n * RBO);
+        }
+    } else {
+        if (valid) store_rec<TO, NV * CO, SO, R>(out, c, acc);
+    }
+}
+
+template <int DIM, int NV, int M, int PREC, int TREE>
+__global__ void __launch_bounds__(128) k_diff_tree(DevMesh mesh, const void *__restrict__ in_v, void *__restrict__ out_v)
+{
+    extern __shared__ __align__(16) unsigned char smo[];
+    diff_cells_tree<DIM, NV, M, PREC, TREE>(mesh, in_v, out_v, (int)(blockIdx.x * blockDim.x + threadIdx.x), threadIdx.x,
+                                            blockDim.x, (long long)blockIdx.x * blockDim.x, smo);
+}
 
 template <int DIM, int NV, int M, int PREC, int LPC>
 __global__ void __launch_bounds__(256) k_diff(DevMesh mesh, const void *__restrict__ in_v, void *__restrict__ out_v)
@@ -719,11 +857,6 @@ __device__ __forceinline__ bool nonfinite32(R x)
     return (__float_as_uint((float)x) & 0x7f800000u) == 0x7f800000u;
 }
 
-// Correctly rounded products and sums that the compiler may not fuse: the increment
-// arithmetic is then the same in every stage kernel, whatever each one inlines.
-__device__ __forceinline__ float mul_rn(float x, float y) { return __fmul_rn(x, y); }
-__device__ __forceinline__ float add_rn(float x, float y) { return __fadd_rn(x, y); }
-
 // Variable v of cell c; r = R_c (residual).  Returns true on NaN/Inf.
 template <class R, class T0, int S0>
 __device__ __forceinline__ bool incr_update(const StageArgs &a, int c, int v, long long n, R r, R dtr, T0 *nxt)
@@ -956,7 +1089,9 @@ __global__ void __launch_bounds__(256) k_flux(DevMesh mesh, StageArgs a)
     for (int v = 0; v < NV; ++v) out[v * nf + f] = F[v];
 }
 
-template <int DIM, int NV, int PREC>
+// TREE 4 or 8: the fluxes are summed in the order of the TREE-lane cell-centric kernel
+// (see diff_cells_tree), whose results the pair then reproduces; 0: in slot order.
+template <int DIM, int NV, int PREC, int TREE>
 __global__ void __launch_bounds__(256) k_gather(DevMesh mesh, StageArgs a)
 {
     using R = typename PrecT<PREC>::R;
@@ -978,7 +1113,33 @@ __global__ void __launch_bounds__(256) k_gather(DevMesh mesh, StageArgs a)
             res[v] += side ? F : -F;
         }
     };
-    if (s1 - s0 == 4 && (s0 & 3) == 0) {
+    if constexpr (TREE > 0) {
+        R F[TREE][NV];
+        const int ns = s1 - s0;
+#pragma unroll
+        for (int l = 0; l < TREE; ++l) {
+#pragma unroll
+            for (int v = 0; v < NV; ++v) F[l][v] = (R)0;
+            if (l < ns) {
+                const unsigned word = __ldg(mesh.sword + s0 + l);
+                const long long f = (long long)(word >> 2);
+#pragma unroll
+                for (int v = 0; v < NV; ++v) {
+                    const R x = __ldg(flux + v * nf + f);
+                    F[l][v] = (word & 1) ? x : -x;
+                }
+            }
+        }
+#pragma unroll
+        for (int o = TREE / 2; o >= 1; o >>= 1)
+#pragma unroll
+            for (int l = 0; l < TREE / 2; ++l)
+                if (l < o)
+#pragma unroll
+                    for (int v = 0; v < NV; ++v) F[l][v] = add_rn(F[l][v], F[l + o][v]);
+#pragma unroll
+        for (int v = 0; v < NV; ++v) res[v] = F[0][v];
+    } else if (s1 - s0 == 4 && (s0 & 3) == 0) {
         // the four slot words of a four-slot cell (tetrahedron, quad): one aligned
         // 16-byte load
         const uint4 w = __ldg(reinterpret_cast<const uint4 *>(mesh.sword + s0));

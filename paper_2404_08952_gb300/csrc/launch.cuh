@@ -12,6 +12,10 @@ namespace dol {
 // block size.
 struct Tune {
     int diff_lpc = 4, diff_block = 256, stage_lpc = 4, stage_block = 128;
+    // 4 or 8: the one-thread-per-cell passes (diff_lpc 1) and the face-centric gather
+    // (stage_lpc -2) sum in the order of that many lanes per cell (cells of at most
+    // `tree` slots, bulk precision below FP64); 0: in slot order
+    int tree = 0;
 };
 
 // Grid of a persistent kernel: resident CTAs per SM x SMs (cached per kernel and
@@ -74,6 +78,23 @@ template <int DIM, int NV, int NS, int PREC> struct Path {
             attr = true;
         }
         k_diff<DIM, NV, MM, PREC, 1><<<nblk(m.n_cells, bs), bs, out_smem<MM>(bs), s>>>(m, in, out);
+    }
+    // one thread per cell, summing in the order of TREE lanes
+    template <int TREE> static void diff_tree(const DevMesh &m, int M, const void *in, void *out, cudaStream_t s)
+    {
+        constexpr int BS = 64;   // its staged output records stay below 48 KB for every order
+        auto go = [&](auto mc) {
+            constexpr int MM = decltype(mc)::value;
+            static_assert(BS * out_rec_bytes<MM>() <= 48 * 1024, "staged records without an opt-in");
+            k_diff_tree<DIM, NV, MM, PREC, TREE><<<nblk(m.n_cells, BS), BS, out_smem<MM>(BS), s>>>(m, in, out);
+        };
+        switch (M) {
+        case 1: go(std::integral_constant<int, 1>{}); break;
+        case 2: go(std::integral_constant<int, 2>{}); break;
+        case 3: go(std::integral_constant<int, 3>{}); break;
+        case 4: go(std::integral_constant<int, 4>{}); break;
+        default: break;
+        }
     }
     template <int LPC> static void diff_l(const DevMesh &m, int M, const void *in, void *out, int bs, cudaStream_t s)
     {
@@ -190,6 +211,10 @@ template <int DIM, int NV, int NS, int PREC> struct Path {
             }
             return;
         }
+        if constexpr (PREC != PREC_F64) {
+            if (t.tree == 4) return diff_tree<4>(m, M, in, out, s);
+            if (t.tree == 8) return diff_tree<8>(m, M, in, out, s);
+        }
         switch (t.diff_lpc) {
         case 4: diff_l<4>(m, M, in, out, t.diff_block, s); break;
         case 8: diff_l<8>(m, M, in, out, t.diff_block, s); break;
@@ -219,7 +244,12 @@ template <int DIM, int NV, int NS, int PREC> struct Path {
     {
         if (t.stage_lpc == -2) {                    // face-centric pair
             k_flux<DIM, NV, NS, PREC><<<nblk(m.n_faces, 128), 128, 0, s>>>(m, a);
-            k_gather<DIM, NV, PREC><<<nblk(m.n_cells, t.stage_block), t.stage_block, 0, s>>>(m, a);
+            const int bs = t.stage_block, nb = nblk(m.n_cells, bs);
+            if constexpr (PREC != PREC_F64) {
+                if (t.tree == 4) return k_gather<DIM, NV, PREC, 4><<<nb, bs, 0, s>>>(m, a);
+                if (t.tree == 8) return k_gather<DIM, NV, PREC, 8><<<nb, bs, 0, s>>>(m, a);
+            }
+            k_gather<DIM, NV, PREC, 0><<<nb, bs, 0, s>>>(m, a);
             return;
         }
         if (t.stage_lpc < 0) {
@@ -311,9 +341,25 @@ inline int path_index(int dim, int nv, int ns, int prec)
 }
 constexpr int N_PATHS = 2 * 2 * 4 * 3;
 
-void register_paths_d2s(PathFns *t);
-void register_paths_d2e(PathFns *t);
-void register_paths_d3s(PathFns *t);
-void register_paths_d3e(PathFns *t);
+// one translation unit per dimension, variable count and precision (compiled in parallel)
+template <int DIM, int NV, int PREC> inline void register_paths(PathFns *t)
+{
+    t[path_index(DIM, NV, 1, PREC)] = Path<DIM, NV, 1, PREC>::fns();
+    t[path_index(DIM, NV, 2, PREC)] = Path<DIM, NV, 2, PREC>::fns();
+    t[path_index(DIM, NV, 3, PREC)] = Path<DIM, NV, 3, PREC>::fns();
+    t[path_index(DIM, NV, 4, PREC)] = Path<DIM, NV, 4, PREC>::fns();
+}
+void register_paths_d2s_f64(PathFns *t);
+void register_paths_d2s_f32(PathFns *t);
+void register_paths_d2s_bf16(PathFns *t);
+void register_paths_d2e_f64(PathFns *t);
+void register_paths_d2e_f32(PathFns *t);
+void register_paths_d2e_bf16(PathFns *t);
+void register_paths_d3s_f64(PathFns *t);
+void register_paths_d3s_f32(PathFns *t);
+void register_paths_d3s_bf16(PathFns *t);
+void register_paths_d3e_f64(PathFns *t);
+void register_paths_d3e_f32(PathFns *t);
+void register_paths_d3e_bf16(PathFns *t);
 
 }  // namespace dol

@@ -1,0 +1,79 @@
+"""The untuned launch shape of larger meshes (one thread per cell, face-centric stage)
+sums in the order of one lane per face slot, so below FP64 it gives the bits of that
+shape, which smaller meshes use and dolinc_set_tuning selects."""
+import numpy as np
+import pytest
+
+import synth
+import paper_2404_08952_gb300 as dg
+
+pytestmark = pytest.mark.gpu
+
+STENCIL = {2: (2, 1), 3: (3, 1), 4: (4, 1), 5: (5, 2)}
+
+
+def _mesh(name):
+    if name == "tri":
+        return synth.tri_mesh(96, 91, jitter=0.2, seed=1)
+    if name == "tri_open":
+        return synth.tri_mesh(101, 83, jitter=0.2, seed=2, boundary="transmissive")
+    if name == "tet":
+        return synth.tet_mesh((16, 14, 16), jitter=0.15, seed=3)
+    if name == "hexprism":
+        return synth.hexprism_mesh((23, 24, 25), jitter=0.2, seed=4)
+    return synth.hex_mesh(np.linspace(0, 1, 27), np.linspace(0, 1, 28), np.linspace(0, 1, 26) ** 1.3,
+                          periodic=(True, True, False))
+
+
+@pytest.mark.parametrize("name,flux,order,n_diff,precision,limiter", [
+    ("tri", "upwind", 3, 2, "fp32", "none"),
+    ("tri", "burgers", 4, 3, "fp32_bf16", "none"),
+    ("tri_open", "rusanov", 3, 2, "fp32", "weno5_all"),
+    ("tri_open", "rusanov", 2, 1, "fp32_bf16", "none"),
+    ("tri_open", "rusanov", 3, 2, "fp32", "eno3_all"),
+    ("tet", "rusanov", 3, 2, "fp32", "none"),
+    ("tet", "rusanov", 4, 3, "fp32_bf16", "eno3_all"),
+    ("tet", "rusanov", 5, 4, "fp32", "none"),
+    ("hexprism", "upwind", 5, 4, "fp32", "none"),
+    ("hexprism", "upwind", 3, 2, "fp32_bf16", "none"),
+    ("hexprism", "rusanov", 3, 2, "fp32", "none"),
+    ("hexprism", "rusanov", 5, 4, "fp32", "none"),
+    ("hex", "rusanov", 4, 3, "fp32", "none"),
+    ("hex", "upwind", 5, 4, "fp32_bf16", "none"),
+])
+def test_untuned_shape_gives_the_lane_shape_bits(name, flux, order, n_diff, precision, limiter):
+    import torch
+    m = _mesh(name)
+    M = dg.Mesh(m)
+    assert M.n_cells >= 16384
+    dim = M.dim
+    nv = dim + 2 if flux == "rusanov" else 1
+    k, r = STENCIL[order]
+    sch = dg.Scheme(k=k, r=r, n_diff=n_diff, flux=flux, nv=nv, precision=precision, limiter=limiter,
+                    adv=(1.0, 0.7, -0.4)[:dim])
+    rng = np.random.default_rng(5)
+    xc = M.geometry()["xc"]
+    s = 0.3 * np.sin(2 * np.pi * xc[:, 0] + 1.0) * np.cos(2 * np.pi * xc[:, 1]) + 0.02 * rng.random(M.n_cells)
+    if nv == 1:
+        u0 = (1.0 + s)[None]
+    else:
+        u0 = np.stack([1.0 + s] + [0.4 + 0.2 * np.roll(s, 7 * d) for d in range(dim)] + [3.0 + 0.5 * s])
+    lanes = 4 if name in ("tri", "tri_open", "tet") else 8
+
+    def run():
+        ws = dg.workspace(M, sch)
+        u = torch.from_numpy(u0).cuda()
+        R = torch.empty_like(u)
+        dg.dolinc_residual(M, sch, u, R, ws)
+        dg.dolinc_rk_steps(M, sch, 1e-3, 2, u, ws)
+        d = torch.zeros(dg.dolinc_diff_layout(M, sch, n_diff)[3] + 256, dtype=torch.uint8, device="cuda")
+        d = d[(-d.data_ptr()) % 256:]
+        dg.dolinc_differentials(M, sch, torch.from_numpy(u0).cuda(), n_diff, d, ws)
+        return [R.cpu().numpy(), u.cpu().numpy()] + dg.diff_to_numpy(M, sch, d, n_diff)
+
+    got = run()
+    dg.dolinc_set_tuning(M, sch, lanes, 256, lanes, 128)
+    want = run()
+    for a, b in zip(got, want):
+        assert np.isfinite(a).all()
+        np.testing.assert_array_equal(a, b)
