@@ -332,7 +332,8 @@ dolinc_status dolinc_indicator_features(dolinc_mesh *mesh, const dolinc_scheme *
  * b3 W4[1][64] b4[1], kept on the device (FP32 master + Adam state); the network
  * computes with their bfloat16 roundings and FP32 accumulation.  Inference runs on
  * the tensor cores (BF16 activations); training runs in FP32 on the same bfloat16
- * weights.  The handle owns its device memory (training scratch grows with the batch). */
+ * weights, with the gradient summed in a fixed order.  The handle owns its device memory
+ * (12 MB of it for partial gradients); training allocates nothing. */
 typedef struct dolinc_mlp dolinc_mlp;
 #define DOLINC_MLP_PARAMS 9985
 dolinc_status dolinc_mlp_create(dolinc_mlp **out, uint64_t seed);       /* He-uniform, zero biases */

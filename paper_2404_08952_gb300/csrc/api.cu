@@ -100,6 +100,7 @@ struct dolinc_mesh {
     int bv_nv = 0;                     // variables of the boundary values set (0: none yet)
     std::vector<int32_t> bidx_h;       // host copy of DevMesh::bidx
     int max_faces = 0;                 // largest number of slots of a cell
+    unsigned *steps_bar = nullptr;     // grid-barrier words of k_steps_small, zero between launches
     std::map<std::string, Tune> tuned;  // launch shapes chosen by dolinc_autotune, per scheme
     // per-kernel timing (dolinc_profile_enable)
     bool prof = false;
@@ -131,25 +132,16 @@ struct dolinc_mesh {
 
 struct dolinc_mlp {
     int device = 0;
-    float *theta = nullptr, *q = nullptr, *m = nullptr, *v = nullptr, *g = nullptr, *loss = nullptr;
+    float *theta = nullptr, *m = nullptr, *v = nullptr, *part = nullptr;
     uint2 *frag = nullptr;
     bool frag_ok = false;
     int step = 0;
-    long long cap = 0;
-    float *A1 = nullptr, *A2 = nullptr, *A3 = nullptr, *z = nullptr, *dZa = nullptr, *dZb = nullptr;
-    void free_scratch()
-    {
-        for (float *p : {A1, A2, A3, z, dZa, dZb}) cudaFree(p);
-        A1 = A2 = A3 = z = dZa = dZb = nullptr;
-        cap = 0;
-    }
     ~dolinc_mlp()
     {
         int cur = 0;
         cudaGetDevice(&cur);
         cudaSetDevice(device);
-        free_scratch();
-        for (void *p : {(void *)theta, (void *)q, (void *)m, (void *)v, (void *)g, (void *)loss, (void *)frag}) cudaFree(p);
+        for (void *p : {(void *)theta, (void *)m, (void *)v, (void *)part, (void *)frag}) cudaFree(p);
         cudaSetDevice(cur);
     }
 };
@@ -361,7 +353,10 @@ std::string scheme_key(const dolinc_mesh *m, const dolinc_scheme *s)
     return k.str();
 }
 
-constexpr int64_t kTreeCells = 16384;
+// From this many cells one thread per cell (and the face-centric stage's extra launch) is
+// no slower than one lane per slot: a step on 20k tetrahedra takes 59 us against 46, on
+// 40k 69 against 67, on 69k 73 against 80; 33k / 65k triangles 55 / 60 us against 49 / 65.
+constexpr int64_t kTreeCells = 40000;
 
 Tune tune_for(const dolinc_mesh *m, const dolinc_scheme *s)
 {
@@ -371,7 +366,9 @@ Tune tune_for(const dolinc_mesh *m, const dolinc_scheme *s)
     const int lanes = m->max_faces <= 4 ? 4 : 8;
     t.diff_lpc = t.stage_lpc = lanes;             // one lane per face slot
     if (s->precision == DOLINC_FP64) {
-        t.diff_lpc = pair_scheme(s) ? 2 : 1;
+        // slot order; unpaired passes (the second runs beside the stage): a step on 69k
+        // tetrahedra takes 352 us, paired 383, one lane per slot 662
+        t.diff_lpc = 1;
         t.diff_block = 64;
         t.stage_lpc = -2;
         t.stage_block = 64;
@@ -610,6 +607,9 @@ dolinc_status upload_mesh(dolinc_mesh *m)
         (st = upload(m, fo, &d.fo)) || (st = upload(m, fn, &d.fn)) || (st = upload(m, fe, &d.face_ext)) ||
         (st = upload(m, ff, &d.face_flip)) || (st = upload(m, fown, &d.fown)))
         return st;
+    const unsigned *bar = nullptr;
+    if ((st = upload(m, std::vector<unsigned>(64, 0u), &bar))) return st;
+    m->steps_bar = const_cast<unsigned *>(bar);
     return DOLINC_OK;
 }
 
@@ -790,6 +790,35 @@ dolinc_status dolinc_rk_stage(dolinc_mesh *m, const dolinc_scheme *s, double dt,
 
 namespace {
 
+// Whole steps of a small mesh in one launch (k_steps_small): untuned calls whose stencil
+// reads order 1 and that compute no order above 2, without Dirichlet/Neumann faces or
+// per-kernel timing.
+constexpr int64_t kSmallCells = 40000;
+bool small_steps_ok(const dolinc_mesh *m, const PathFns *p, const dolinc_scheme *s)
+{
+    return p->steps_small && s->n_diff <= 2 && m->h.n_cells <= kSmallCells && m->max_faces <= 8 && m->d.n_bcell == 0 &&
+           !m->prof && !m->part && !m->tuned.count(scheme_key(m, s));
+}
+
+cudaError_t small_steps(dolinc_mesh *m, const PathFns *p, const dolinc_scheme *s, double dt, double *u, void *ws,
+                        const WsLayout &L, cudaStream_t cs, int n_steps)
+{
+    StepsArgs q{};
+    q.a = base_args(m, s, ws, L, L.o0[0]);
+    q.a.dt = dt;
+    q.a.dacc = reinterpret_cast<float *>(B(ws, L.dacc));
+    q.u = u;
+    q.ust = reinterpret_cast<double *>(B(ws, L.ustage));
+    for (int i = 0; i < 3; ++i) q.o0[i] = B(ws, L.o0[i]);
+    q.ord1 = B(ws, L.ord[1]);
+    q.ord2 = B(ws, L.ord[2]);
+    q.n_diff = s->n_diff;
+    q.n_steps = n_steps;
+    q.bar = m->steps_bar;
+    q.spin_limit = 1u << 22;
+    return p->steps_small(m->d, q, m->max_faces <= 4 ? 4 : 8, cs);
+}
+
 // One SSP-RK3 step.  The first kernel reads the step's state from u_in and, when
 // u_dev differs from it, also writes it to u_dev; the stages read the step's start
 // state from u_dev; the last stage writes the new state to u_out.  dolinc_rk_step
@@ -800,6 +829,10 @@ dolinc_status rk_step_impl(dolinc_mesh *m, const dolinc_scheme *s, double dt, co
     static const double A[3] = {0.0, 0.75, 1.0 / 3.0}, Bc[3] = {1.0, 0.25, 2.0 / 3.0};
     const PathFns *p = path_for(m, s, needed_order(*s));
     if (!p) return fail(DOLINC_ERR_UNSUPPORTED, "no kernel for this (dim, nv, order, precision)");
+    if (u_in == u_dev && u_out == u_dev && small_steps_ok(m, p, s)) {
+        if (small_steps(m, p, s, dt, u_dev, ws, L, cs, n_steps) == cudaSuccess) return launch_check();
+        cudaGetLastError();                       // no room for a cooperative grid: separate launches
+    }
     double *ust = reinterpret_cast<double *>(B(ws, L.ustage));
     const Tune tn = tune_for(m, s);
     // Several steps in one call keep the state on the device: the last stage of a step
@@ -1135,47 +1168,6 @@ uint64_t splitmix(uint64_t &x)
     z = (z ^ (z >> 27)) * 0x94D049BB133111EBULL;
     return z ^ (z >> 31);
 }
-
-dolinc_status mlp_scratch(dolinc_mlp *m, long long n)
-{
-    if (n <= m->cap) return DOLINC_OK;
-    m->free_scratch();
-    const size_t h = sizeof(float) * (size_t)n * MLP_H;
-    CU(cudaMalloc(&m->A1, h));
-    CU(cudaMalloc(&m->A2, h));
-    CU(cudaMalloc(&m->A3, h));
-    CU(cudaMalloc(&m->z, sizeof(float) * (size_t)n));
-    CU(cudaMalloc(&m->dZa, h));
-    CU(cudaMalloc(&m->dZb, h));
-    m->cap = n;
-    return DOLINC_OK;
-}
-
-// loss and gradient of one batch into m->g (and *loss_dev); forward on the bf16 weights
-dolinc_status mlp_grad(dolinc_mlp *m, const float *x, const uint8_t *y, long long n, float pw, float *loss_dev,
-                       cudaStream_t cs)
-{
-    dolinc_status st = mlp_scratch(m, n);
-    if (st) return st;
-    const float *q = m->q;
-    launch_quantize(m->theta, m->q, cs);
-    launch_dense_fwd(x, MLP_IN, q + OFF_W1, q + OFF_B1, MLP_H, n, m->A1, true, cs);
-    launch_dense_fwd(m->A1, MLP_H, q + OFF_W2, q + OFF_B2, MLP_H, n, m->A2, true, cs);
-    launch_dense_fwd(m->A2, MLP_H, q + OFF_W3, q + OFF_B3, MLP_H, n, m->A3, true, cs);
-    launch_dense_fwd(m->A3, MLP_H, q + OFF_W4, q + OFF_B4, 1, n, m->z, false, cs);
-    CU(cudaMemsetAsync(m->g, 0, sizeof(float) * MLP_PARAMS, cs));
-    if (loss_dev) CU(cudaMemsetAsync(loss_dev, 0, sizeof(float), cs));
-    float *dz = m->dZa;
-    launch_bce(m->z, y, n, pw, dz, loss_dev, cs);
-    launch_dense_bwd_w(dz, m->A3, MLP_H, 1, n, m->g + OFF_W4, m->g + OFF_B4, cs);
-    launch_dense_bwd_x(dz, q + OFF_W4, MLP_H, 1, n, m->A3, m->dZb, cs);              // dZ3
-    launch_dense_bwd_w(m->dZb, m->A2, MLP_H, MLP_H, n, m->g + OFF_W3, m->g + OFF_B3, cs);
-    launch_dense_bwd_x(m->dZb, q + OFF_W3, MLP_H, MLP_H, n, m->A2, m->dZa, cs);     // dZ2
-    launch_dense_bwd_w(m->dZa, m->A1, MLP_H, MLP_H, n, m->g + OFF_W2, m->g + OFF_B2, cs);
-    launch_dense_bwd_x(m->dZa, q + OFF_W2, MLP_H, MLP_H, n, m->A1, m->dZb, cs);     // dZ1
-    launch_dense_bwd_w(m->dZb, x, MLP_IN, MLP_H, n, m->g + OFF_W1, m->g + OFF_B1, cs);
-    return launch_check();
-}
 }  // namespace
 
 dolinc_status dolinc_criterion(dolinc_mesh *m, const dolinc_scheme *s, const double *u, uint8_t *flags, double kappa,
@@ -1227,9 +1219,9 @@ dolinc_status dolinc_mlp_create(dolinc_mlp **out, uint64_t seed)
     }
     auto al = [&](void **p, size_t b) { return cudaMalloc(p, b); };
     cudaError_t e = cudaSuccess;
-    for (float **p : {&m->theta, &m->q, &m->m, &m->v, &m->g})
+    for (float **p : {&m->theta, &m->m, &m->v})
         if (e == cudaSuccess) e = al((void **)p, sizeof(float) * MLP_PARAMS);
-    if (e == cudaSuccess) e = al((void **)&m->loss, sizeof(float));
+    if (e == cudaSuccess) e = al((void **)&m->part, sizeof(float) * MLP_PART * MLP_MAX_PARTS);
     if (e == cudaSuccess) e = al((void **)&m->frag, sizeof(uint2) * N_FRAGS * 32);
     if (e == cudaSuccess) e = cudaMemcpy(m->theta, th.data(), sizeof(float) * MLP_PARAMS, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemset(m->m, 0, sizeof(float) * MLP_PARAMS);
@@ -1278,10 +1270,9 @@ dolinc_status dolinc_mlp_loss_grad(dolinc_mlp *m, const float *x, const uint8_t 
 {
     if (!m || !x || !y || n <= 0) return fail(DOLINC_ERR_INVALID_ARG, "bad argument");
     cudaStream_t cs = reinterpret_cast<cudaStream_t>(stream);
-    dolinc_status st = mlp_grad(m, x, y, n, pos_weight, loss, cs);
-    if (st) return st;
-    if (grad) CU(cudaMemcpyAsync(grad, m->g, sizeof(float) * MLP_PARAMS, cudaMemcpyDeviceToDevice, cs));
-    return DOLINC_OK;
+    const int np = launch_mlp_grad(m->theta, x, y, n, pos_weight, m->part, cs);
+    launch_mlp_reduce(m->part, np, grad, loss, nullptr, nullptr, nullptr, 0.f, 1, cs);
+    return launch_check();
 }
 
 dolinc_status dolinc_mlp_train_step(dolinc_mlp *m, const float *x, const uint8_t *y, int64_t n, float lr,
@@ -1289,10 +1280,9 @@ dolinc_status dolinc_mlp_train_step(dolinc_mlp *m, const float *x, const uint8_t
 {
     if (!m || !x || !y || n <= 0) return fail(DOLINC_ERR_INVALID_ARG, "bad argument");
     cudaStream_t cs = reinterpret_cast<cudaStream_t>(stream);
-    dolinc_status st = mlp_grad(m, x, y, n, pos_weight, loss, cs);
-    if (st) return st;
+    const int np = launch_mlp_grad(m->theta, x, y, n, pos_weight, m->part, cs);
     m->step += 1;
-    launch_adam(m->theta, m->m, m->v, m->g, MLP_PARAMS, lr, m->step, cs);
+    launch_mlp_reduce(m->part, np, nullptr, loss, m->theta, m->m, m->v, lr, m->step, cs);
     m->frag_ok = false;
     return launch_check();
 }

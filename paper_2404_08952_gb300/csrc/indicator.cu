@@ -348,81 +348,257 @@ __global__ void __launch_bounds__(128) k_mlp_infer(const uint2 *__restrict__ fra
 }
 
 // ------------------------------------------------------------------ training (FP32)
-__global__ void k_quantize(const float *__restrict__ theta, float *__restrict__ q, int n)
+// Loss and gradient of a minibatch in two launches.
+//
+// k_mlp_grad: a CTA takes tiles of 64 rows through the forward and the backward pass with
+// every activation in shared memory and adds the tile's weight gradient to 4 x 4 register
+// blocks, one per thread and layer; after its last tile it writes one partial gradient.
+// k_mlp_reduce sums the partials in CTA order (the gradient does not depend on which CTA
+// finishes first) and, for a training step, applies Adam to the sum.
+// Bound: FP32 FMA, 29 k per row (8192 rows: 3 us of the chip's FMA rate; one 64-row tile
+// takes one CTA about 10 us, which is what a minibatch of up to 304 tiles costs).
+// One kernel per layer and operand (a thread per output element, every activation through
+// memory, weight gradients by serial loops over 2048 rows on 4 to 132 blocks, added
+// atomically) took 1242 us at 8192 rows.
+// Rows of 64 activations are 68 floats apart, rows of 24 inputs 28: eight consecutive
+// rows' 16-byte pieces then lie in distinct banks.
+constexpr int GT = 64, LDH = 68, LDX = 28;
+struct MlpTile {
+    float w1[MLP_H][LDX], w2[MLP_H][LDH], w3[MLP_H][LDH], w4[MLP_H], b[3][MLP_H], b4[4];
+    float x[GT][LDX], h1[GT][LDH], h2[GT][LDH], h3[GT][LDH], dz[GT], loss[GT];
+};
+
+__device__ __forceinline__ float bf16_round(float x) { return __bfloat162float(__float2bfloat16_rn(x)); }
+__device__ __forceinline__ float4 lds4(const float *p) { return *reinterpret_cast<const float4 *>(p); }
+__device__ __forceinline__ void fma4(float (&c)[4], float a, float4 b)
 {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) q[i] = __bfloat162float(__float2bfloat16_rn(theta[i]));
+    c[0] = fmaf(a, b.x, c[0]), c[1] = fmaf(a, b.y, c[1]), c[2] = fmaf(a, b.z, c[2]), c[3] = fmaf(a, b.w, c[3]);
+}
+__device__ __forceinline__ float dot4(float4 a, float4 b, float c)
+{
+    return fmaf(a.w, b.w, fmaf(a.z, b.z, fmaf(a.y, b.y, fmaf(a.x, b.x, c))));
 }
 
-// Z[r][o] = b[o] + sum_i A[r][i] W[o][i]  (ReLU on request); one thread per (r, o)
-__global__ void k_dense_fwd(const float *__restrict__ A, int in_dim, const float *__restrict__ W,
-                            const float *__restrict__ b, int out_dim, long long n, float *__restrict__ Z, int relu)
+// out[r][o] = relu(b[o] + sum_k in[r][k] w[o][k]): rows 4 ty.., columns tx + 16 j
+template <int K, int LDI, int LDW>
+__device__ __forceinline__ void tile_forward(const float (*in)[LDI], const float (*w)[LDW], const float *b,
+                                             float (*out)[LDH], int ty, int tx)
 {
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n * out_dim) return;
-    const long long r = i / out_dim;
-    const int o = (int)(i % out_dim);
-    float s = b[o];
-    for (int k = 0; k < in_dim; ++k) s = fmaf(A[r * in_dim + k], W[o * in_dim + k], s);
-    Z[i] = relu ? fmaxf(s, 0.f) : s;
-}
-
-// dW[o][i] += sum_r dZ[r][o] A[r][i], db[o] += sum_r dZ[r][o]: one thread per (o, i | bias)
-// and chunk of rows, atomically added (the weight gradient is a small dense array).
-__global__ void k_dense_bwd_w(const float *__restrict__ dZ, const float *__restrict__ A, int in_dim, int out_dim,
-                              long long n, float *__restrict__ dW, float *__restrict__ db, int chunk)
-{
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    const int per = in_dim + 1;
-    if (j >= out_dim * per) return;
-    const int o = j / per, i = j % per;
-    const long long r0 = (long long)blockIdx.y * chunk;
-    const long long r1 = r0 + chunk < n ? r0 + chunk : n;
-    float s = 0.f;
-    for (long long r = r0; r < r1; ++r) s = fmaf(dZ[r * out_dim + o], i < in_dim ? A[r * in_dim + i] : 1.f, s);
-    if (i < in_dim) atomicAdd(dW + o * in_dim + i, s);
-    else atomicAdd(db + o, s);
-}
-
-// dA[r][i] = (sum_o dZ[r][o] W[o][i]) * (Amask[r][i] > 0)
-__global__ void k_dense_bwd_x(const float *__restrict__ dZ, const float *__restrict__ W, int in_dim, int out_dim,
-                              long long n, const float *__restrict__ Amask, float *__restrict__ dA)
-{
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n * in_dim) return;
-    const long long r = i / in_dim;
-    const int k = (int)(i % in_dim);
-    float s = 0.f;
-    for (int o = 0; o < out_dim; ++o) s = fmaf(dZ[r * out_dim + o], W[o * in_dim + k], s);
-    dA[i] = Amask[i] > 0.f ? s : 0.f;
-}
-
-// weighted BCE with logits: dz = (s (pw y + 1 - y) - pw y) / n, loss summed into *loss
-__global__ void k_bce(const float *__restrict__ z, const uint8_t *__restrict__ y, long long n, float pw,
-                      float *__restrict__ dz, float *__restrict__ loss)
-{
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    float l = 0.f;
-    if (i < n) {
-        const float zi = z[i], yi = y[i] ? 1.f : 0.f;
-        const float s = 1.f / (1.f + expf(-zi));
-        dz[i] = (s * (pw * yi + 1.f - yi) - pw * yi) / (float)n;
-        const float lsp = zi > 0.f ? zi + log1pf(expf(-zi)) : log1pf(expf(zi));   // log(1 + e^z)
-        l = (pw * yi * (lsp - zi) + (1.f - yi) * lsp) / (float)n;
+    float c[4][4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) c[i][j] = b[tx + 16 * j];
+#pragma unroll 2
+    for (int k = 0; k < K; k += 4) {
+        float4 a[4], q[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) a[i] = lds4(&in[4 * ty + i][k]);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) q[j] = lds4(&w[tx + 16 * j][k]);
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) c[i][j] = dot4(a[i], q[j], c[i][j]);
     }
-    for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
-    if ((threadIdx.x & 31) == 0 && loss) atomicAdd(loss, l);
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) out[4 * ty + i][tx + 16 * j] = fmaxf(c[i][j], 0.f);
 }
 
-__global__ void k_adam(float *theta, float *m, float *v, const float *g, int n, float lr, float c1, float c2)
+// d[o][k] += sum_r dz[r][o] h[r][k]: rows o = 4 ty.., columns k = 4 tx..
+template <int LDI>
+__device__ __forceinline__ void tile_grad(const float (*dz)[LDH], const float (*h)[LDI], float (&d)[4][4], int ty, int tx)
 {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const float gi = g[i];
-    const float mi = 0.9f * m[i] + 0.1f * gi, vi = 0.999f * v[i] + 0.001f * gi * gi;
-    m[i] = mi;
-    v[i] = vi;
-    theta[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + 1e-8f);
+#pragma unroll 4
+    for (int r = 0; r < GT; ++r) {
+        const float4 a = lds4(&dz[r][4 * ty]), q = lds4(&h[r][4 * tx]);
+        fma4(d[0], a.x, q);
+        fma4(d[1], a.y, q);
+        fma4(d[2], a.z, q);
+        fma4(d[3], a.w, q);
+    }
+}
+
+// h[r][k] <- (h[r][k] > 0) sum_o dz[r][o] w[o][k], in place (ends with a barrier)
+__device__ __forceinline__ void tile_backward(const float (*dz)[LDH], const float (*w)[LDH], float (*h)[LDH], int ty,
+                                              int tx)
+{
+    float c[4][4] = {};
+#pragma unroll 2
+    for (int o = 0; o < MLP_H; o += 4) {
+        float4 a[4], q[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) a[i] = lds4(&dz[4 * ty + i][o]);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) q[j] = lds4(&w[o + j][4 * tx]);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            fma4(c[i], a[i].x, q[0]);
+            fma4(c[i], a[i].y, q[1]);
+            fma4(c[i], a[i].z, q[2]);
+            fma4(c[i], a[i].w, q[3]);
+        }
+    }
+    __syncthreads();                              // h was also read as the layer's input
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        float4 m = lds4(&h[4 * ty + i][4 * tx]);
+        m.x = m.x > 0.f ? c[i][0] : 0.f, m.y = m.y > 0.f ? c[i][1] : 0.f;
+        m.z = m.z > 0.f ? c[i][2] : 0.f, m.w = m.w > 0.f ? c[i][3] : 0.f;
+        *reinterpret_cast<float4 *>(&h[4 * ty + i][4 * tx]) = m;
+    }
+    __syncthreads();
+}
+
+__device__ __forceinline__ float column_sum(const float (*z)[LDH], int o)
+{
+    float s = 0.f;
+#pragma unroll 8
+    for (int r = 0; r < GT; ++r) s += z[r][o];
+    return s;
+}
+
+__global__ void __launch_bounds__(256) k_mlp_grad(const float *__restrict__ theta, const float *__restrict__ x,
+                                                  const uint8_t *__restrict__ y, long long n, float pw,
+                                                  float *__restrict__ part)
+{
+    extern __shared__ __align__(16) unsigned char raw[];
+    MlpTile &t = *reinterpret_cast<MlpTile *>(raw);
+    const int tid = threadIdx.x, ty = tid / 16, tx = tid % 16;
+    for (int i = tid; i < MLP_H * MLP_IN; i += 256) t.w1[i / MLP_IN][i % MLP_IN] = bf16_round(theta[OFF_W1 + i]);
+    for (int i = tid; i < MLP_H * MLP_H; i += 256) {
+        t.w2[i / MLP_H][i % MLP_H] = bf16_round(theta[OFF_W2 + i]);
+        t.w3[i / MLP_H][i % MLP_H] = bf16_round(theta[OFF_W3 + i]);
+    }
+    if (tid < MLP_H) {
+        t.w4[tid] = bf16_round(theta[OFF_W4 + tid]);
+        t.b[0][tid] = bf16_round(theta[OFF_B1 + tid]);
+        t.b[1][tid] = bf16_round(theta[OFF_B2 + tid]);
+        t.b[2][tid] = bf16_round(theta[OFF_B3 + tid]);
+    }
+    if (tid == 0) t.b4[0] = bf16_round(theta[OFF_B4]);
+    float d3[4][4] = {}, d2[4][4] = {}, d1[4][4] = {};
+    float dv = 0.f, db1 = 0.f;                    // thread's bias and output-layer sums, see below
+    const int o = tid % MLP_H, part4 = tid / MLP_H;
+    for (long long r0 = (long long)blockIdx.x * GT; r0 < n; r0 += (long long)gridDim.x * GT) {
+        __syncthreads();
+        for (int i = tid; i < GT * MLP_IN; i += 256) {
+            const long long g = r0 * MLP_IN + i;
+            t.x[i / MLP_IN][i % MLP_IN] = g < n * MLP_IN ? __ldg(x + g) : 0.f;
+        }
+        __syncthreads();
+        tile_forward<MLP_IN, LDX, LDX>(t.x, t.w1, t.b[0], t.h1, ty, tx);
+        __syncthreads();
+        tile_forward<MLP_H, LDH, LDH>(t.h1, t.w2, t.b[1], t.h2, ty, tx);
+        __syncthreads();
+        tile_forward<MLP_H, LDH, LDH>(t.h2, t.w3, t.b[2], t.h3, ty, tx);
+        __syncthreads();
+        {
+            // logit of row tid / 4 by four threads, then the weighted BCE with logits:
+            // dz = (s (pw y + 1 - y) - pw y) / n
+            const int r = tid / 4, q = tid % 4;
+            float z = 0.f;
+#pragma unroll
+            for (int k = 0; k < MLP_H; k += 16) z = dot4(lds4(&t.h3[r][k + 4 * q]), lds4(&t.w4[k + 4 * q]), z);
+            z += __shfl_xor_sync(0xffffffffu, z, 1);
+            z += __shfl_xor_sync(0xffffffffu, z, 2);
+            if (q == 0) {
+                float dz = 0.f, l = 0.f;
+                if (r0 + r < n) {
+                    const float zi = z + t.b4[0], yi = y[r0 + r] ? 1.f : 0.f;
+                    const float s = 1.f / (1.f + expf(-zi));
+                    dz = (s * (pw * yi + 1.f - yi) - pw * yi) / (float)n;
+                    const float lsp = zi > 0.f ? zi + log1pf(expf(-zi)) : log1pf(expf(zi));   // log(1 + e^z)
+                    l = (pw * yi * (lsp - zi) + (1.f - yi) * lsp) / (float)n;
+                }
+                t.dz[r] = dz;
+                t.loss[r] = l;
+            }
+        }
+        __syncthreads();
+        // output layer: threads 0-63 its weights, 64 its bias, 65 the loss
+        if (part4 == 0) {
+#pragma unroll 8
+            for (int r = 0; r < GT; ++r) dv = fmaf(t.dz[r], t.h3[r][o], dv);
+        } else if (tid == 64 || tid == 65) {
+            const float *v = tid == 64 ? t.dz : t.loss;
+#pragma unroll 8
+            for (int r = 0; r < GT; ++r) dv += v[r];
+        }
+        __syncthreads();
+        for (int i = tid; i < GT * MLP_H / 4; i += 256) {        // h3 <- dZ3
+            const int r = i / 16, k = 4 * (i % 16);
+            const float4 h = lds4(&t.h3[r][k]), w = lds4(&t.w4[k]);
+            const float g = t.dz[r];
+            *reinterpret_cast<float4 *>(&t.h3[r][k]) = make_float4(h.x > 0.f ? g * w.x : 0.f, h.y > 0.f ? g * w.y : 0.f,
+                                                                   h.z > 0.f ? g * w.z : 0.f, h.w > 0.f ? g * w.w : 0.f);
+        }
+        __syncthreads();
+        tile_grad<LDH>(t.h3, t.h2, d3, ty, tx);
+        tile_backward(t.h3, t.w3, t.h2, ty, tx);                 // h2 <- dZ2
+        tile_grad<LDH>(t.h2, t.h1, d2, ty, tx);
+        tile_backward(t.h2, t.w2, t.h1, ty, tx);                 // h1 <- dZ1
+        // input layer: 96 threads its weights (16 x 6 blocks of 4 x 4), the others the
+        // biases of the three hidden layers (two threads of 128 take two columns)
+        if (tid < 96) tile_grad<LDX>(t.h1, t.x, d1, tid / 6, tid % 6);
+        else if (tid < 224) {
+            const int q = tid - 96;
+            if (q < 64) db1 += column_sum(t.h1, q);
+            else db1 += column_sum(t.h2, q - 64);
+        }
+        if (tid >= 192 && tid < 256) dv += column_sum(t.h3, tid - 192);
+    }
+    float *g = part + (long long)blockIdx.x * MLP_PART;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const int k = (4 * ty + i) * MLP_H + 4 * tx;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            g[OFF_W3 + k + j] = d3[i][j];
+            g[OFF_W2 + k + j] = d2[i][j];
+        }
+        if (tid < 96)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) g[OFF_W1 + (4 * (tid / 6) + i) * MLP_IN + 4 * (tid % 6) + j] = d1[i][j];
+    }
+    if (part4 == 0) g[OFF_W4 + o] = dv;
+    if (tid == 64) g[OFF_B4] = dv;
+    if (tid == 65) g[MLP_PARAMS] = dv;
+    if (tid >= 96 && tid < 160) g[OFF_B1 + tid - 96] = db1;
+    if (tid >= 160 && tid < 224) g[OFF_B2 + tid - 160] = db1;
+    if (tid >= 192) g[OFF_B3 + tid - 192] = dv;
+}
+
+// Sum of the n_part partials of each parameter (32 parameters x 8 groups of partials per
+// block, each group and then the groups in order); the sum goes to grad, the loss to
+// *loss, and with theta the parameter takes an Adam step (c1, c2: 1 - beta^step).
+__global__ void __launch_bounds__(256) k_mlp_reduce(const float *__restrict__ part, int n_part, float *grad, float *loss,
+                                                    float *theta, float *m, float *v, float lr, float c1, float c2)
+{
+    __shared__ float sh[8][32];
+    const int l = threadIdx.x & 31, w = threadIdx.x >> 5, i = blockIdx.x * 32 + l;
+    float s = 0.f;
+    if (i <= MLP_PARAMS)
+#pragma unroll 8
+        for (int p = w; p < n_part; p += 8) s += __ldg(part + (long long)p * MLP_PART + i);
+    sh[w][l] = s;
+    __syncthreads();
+    if (w != 0 || i > MLP_PARAMS) return;
+#pragma unroll
+    for (int q = 1; q < 8; ++q) s += sh[q][l];
+    if (i == MLP_PARAMS) {
+        if (loss) *loss = s;
+        return;
+    }
+    if (grad) grad[i] = s;
+    if (theta) {
+        const float mi = 0.9f * m[i] + 0.1f * s, vi = 0.999f * v[i] + 0.001f * s * s;
+        m[i] = mi;
+        v[i] = vi;
+        theta[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + 1e-8f);
+    }
 }
 
 template <int DIM, int NSR, int PREC>
@@ -481,35 +657,24 @@ void launch_mlp_infer_fused(const uint2 *frag, const float *theta, const DevMesh
     if (blocks < 1) blocks = 1;
     k_mlp_infer<true><<<blocks, 128, 0, s>>>(frag, theta, nullptr, n, logits, flags, m, own);
 }
-void launch_quantize(const float *theta, float *q, cudaStream_t s)
+int launch_mlp_grad(const float *theta, const float *x, const uint8_t *y, long long n, float pw, float *part,
+                    cudaStream_t s)
 {
-    k_quantize<<<nblk(MLP_PARAMS, 256), 256, 0, s>>>(theta, q, MLP_PARAMS);
+    static bool attr = false;   // opt in to more than 48 KB once
+    if (!attr) {
+        cudaFuncSetAttribute(k_mlp_grad, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(MlpTile));
+        attr = true;
+    }
+    const long long tiles = (n + GT - 1) / GT;
+    const int grid = (int)(tiles < MLP_MAX_PARTS ? tiles : MLP_MAX_PARTS);
+    k_mlp_grad<<<grid, 256, sizeof(MlpTile), s>>>(theta, x, y, n, pw, part);
+    return grid;
 }
-void launch_dense_fwd(const float *A, int in_dim, const float *W, const float *b, int out_dim, long long n, float *Z,
-                      bool relu, cudaStream_t s)
-{
-    k_dense_fwd<<<nblk(n * out_dim, 256), 256, 0, s>>>(A, in_dim, W, b, out_dim, n, Z, relu ? 1 : 0);
-}
-void launch_dense_bwd_w(const float *dZ, const float *A, int in_dim, int out_dim, long long n, float *dW, float *db,
-                        cudaStream_t s)
-{
-    const int chunk = 2048;
-    dim3 grid(nblk(out_dim * (in_dim + 1), 128), (unsigned)((n + chunk - 1) / chunk));
-    k_dense_bwd_w<<<grid, 128, 0, s>>>(dZ, A, in_dim, out_dim, n, dW, db, chunk);
-}
-void launch_dense_bwd_x(const float *dZ, const float *W, int in_dim, int out_dim, long long n, const float *Amask,
-                        float *dA, cudaStream_t s)
-{
-    k_dense_bwd_x<<<nblk(n * in_dim, 256), 256, 0, s>>>(dZ, W, in_dim, out_dim, n, Amask, dA);
-}
-void launch_bce(const float *z, const uint8_t *y, long long n, float pw, float *dz, float *loss, cudaStream_t s)
-{
-    k_bce<<<nblk(n, 256), 256, 0, s>>>(z, y, n, pw, dz, loss);
-}
-void launch_adam(float *theta, float *m, float *v, const float *g, int n, float lr, int step, cudaStream_t s)
+void launch_mlp_reduce(const float *part, int n_part, float *grad, float *loss, float *theta, float *m, float *v,
+                       float lr, int step, cudaStream_t s)
 {
     const float c1 = 1.f - powf(0.9f, (float)step), c2 = 1.f - powf(0.999f, (float)step);
-    k_adam<<<nblk(n, 256), 256, 0, s>>>(theta, m, v, g, n, lr, c1, c2);
+    k_mlp_reduce<<<nblk(MLP_PARAMS + 1, 32), 256, 0, s>>>(part, n_part, grad, loss, theta, m, v, lr, c1, c2);
 }
 
 }  // namespace dol

@@ -35,15 +35,13 @@ void launch_mlp_infer(const uint2 *frag, const float *theta, const float *x, lon
 // the network on every cell of m, its inputs gathered from the own features inside the kernel
 void launch_mlp_infer_fused(const uint2 *frag, const float *theta, const DevMesh &m, const float *own, float *logits,
                             uint8_t *flags, cudaStream_t s);
-void launch_quantize(const float *theta, float *theta_q, cudaStream_t s);
-void launch_dense_fwd(const float *A, int in_dim, const float *W, const float *b, int out_dim, long long n, float *Z,
-                      bool relu, cudaStream_t s);
-void launch_dense_bwd_w(const float *dZ, const float *A, int in_dim, int out_dim, long long n, float *dW, float *db,
-                        cudaStream_t s);
-void launch_dense_bwd_x(const float *dZ, const float *W, int in_dim, int out_dim, long long n, const float *Amask,
-                        float *dA, cudaStream_t s);
-void launch_bce(const float *z, const uint8_t *y, long long n, float pos_weight, float *dz, float *loss,
-                cudaStream_t s);
-void launch_adam(float *theta, float *m, float *v, const float *g, int n, float lr, int step, cudaStream_t s);
+// Partial gradients of a minibatch (one per CTA, MLP_PART floats: the parameters, then the
+// loss; at most MLP_MAX_PARTS) into part; returns their number.  Then their sum, into
+// grad and *loss where not null, and with theta an Adam step on theta, m and v.
+constexpr int MLP_PART = 9988, MLP_MAX_PARTS = 304;      // 304: two CTAs on each of 152 SMs
+int launch_mlp_grad(const float *theta, const float *x, const uint8_t *y, long long n, float pos_weight, float *part,
+                    cudaStream_t s);
+void launch_mlp_reduce(const float *part, int n_part, float *grad, float *loss, float *theta, float *m, float *v,
+                       float lr, int step, cudaStream_t s);
 
 }  // namespace dol

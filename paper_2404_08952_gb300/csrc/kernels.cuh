@@ -161,7 +161,9 @@ DOL_HD constexpr int diff_batch(int rec_values) { return rec_values <= 8 ? 4 : (
 // One differential pass over a group of nt threads (thread t of the group, global
 // thread index gt of the pass; for LPC = 1 the group's cells start at c0 and its
 // output records are staged in smo and written by thread 0 with one bulk copy).
-template <int DIM, int NV, int M, int PREC, int LPC, int UBF = 0>
+// LDG: the input records through the read-only path; else coherent loads (a launch that
+// also writes them).
+template <int DIM, int NV, int M, int PREC, int LPC, int UBF = 0, bool LDG = true>
 __device__ __forceinline__ void diff_cells(const DevMesh &mesh, const void *__restrict__ in_v, void *__restrict__ out_v,
                                            long long gt, int t, int nt, long long c0, unsigned char *smo)
 {
@@ -230,14 +232,14 @@ __device__ __forceinline__ void diff_cells(const DevMesh &mesh, const void *__re
             R x[NV * CI];
             R wx, wy, wz, iv;
             ld4<R>(Geo<R>::cellk(mesh) + 4ll * c, wx, wy, wz, iv);
-            load_rec<TI, NV * CI, SI, R>(in, c, x);
+            load_rec<TI, NV * CI, SI, R, LDG>(in, c, x);
             poly_mul_acc<DIM, NV, M, R>(acc, x, wx, wy, wz);
         }
         for (int s = s0 + l; s < s1; s += LPC * UB) {
             R xs[UB][NV * CI];
 #pragma unroll
             for (int u = 0; u < UB; ++u)
-                if (ok[u]) load_rec<TI, NV * CI, SI, R>(in, nbv[u], xs[u]);
+                if (ok[u]) load_rec<TI, NV * CI, SI, R, LDG>(in, nbv[u], xs[u]);
             R cx[UB], cy[UB], cz[UB];
             bool cok[UB];
 #pragma unroll
@@ -921,11 +923,10 @@ __device__ __forceinline__ bool incr_update_cell(const StageArgs &a, int c, long
 
 // LPC lanes per cell: lane l evaluates slots l, l+LPC, ...; the group sums the signed
 // fluxes by recursive halving and lane l then updates variables [l*B, (l+1)*B).
-template <int DIM, int NV, int NS, int PREC, int LPC>
-__global__ void __launch_bounds__(256, (PREC != PREC_F64 && NS <= 1) ? 4 : 1) k_stage(DevMesh mesh, StageArgs a)
+template <int DIM, int NV, int NS, int PREC, int LPC, class Src>
+__device__ __forceinline__ void stage_lanes(const DevMesh &mesh, const StageArgs &a, const Src &src, long long gt)
 {
     using R = typename PrecT<PREC>::R;
-    const long long gt = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     const int c = (int)(gt / LPC), l = (int)(gt % LPC);
     const bool valid = c < mesh.n_cells;
     constexpr int P = ((NV + LPC - 1) / LPC) * LPC;
@@ -936,7 +937,6 @@ __global__ void __launch_bounds__(256, (PREC != PREC_F64 && NS <= 1) ? 4 : 1) k_
         int s0, s1;
         slot_range(mesh, c, s0, s1);
         const bool own_flag = a.flags && a.flags[c];
-        GlobalSrc<DIM, NV, PREC> src{a, mesh};
 #pragma unroll 2
         for (int s = s0 + l; s < s1; s += LPC) {
             R F[NV];
@@ -980,6 +980,13 @@ __global__ void __launch_bounds__(256, (PREC != PREC_F64 && NS <= 1) ? 4 : 1) k_
         }
     }
     if (bad) atomicOr(a.status, 1u);
+}
+
+template <int DIM, int NV, int NS, int PREC, int LPC>
+__global__ void __launch_bounds__(256, (PREC != PREC_F64 && NS <= 1) ? 4 : 1) k_stage(DevMesh mesh, StageArgs a)
+{
+    GlobalSrc<DIM, NV, PREC> src{a, mesh};
+    stage_lanes<DIM, NV, NS, PREC, LPC>(mesh, a, src, (long long)blockIdx.x * blockDim.x + threadIdx.x);
 }
 
 // Residual R_c = res / V_c and the stage output of one cell (one thread per cell):
@@ -1451,6 +1458,109 @@ __global__ void __launch_bounds__(256) k_batch_stage(DevMesh mesh, StageArgs a, 
         }
         if (nxt) store_rec<T0, NV, S0, R>(nxt, c, o32);
         if (bad) atomicOr(a.status, 1u);
+    }
+}
+
+// ------------------------------------------------------------------ persistent steps of small meshes
+// All stages of n_steps SSP-RK3 steps in one cooperative launch, LPC lanes per cell as
+// k_diff and k_stage run them (the same device code, so below FP64 the same bits).
+// Phases, separated by a grid barrier: pack | order 1 | stage and order 2 | order 1 | ..
+// (order 2 is read by nothing in the stage, so it runs beside it on other warps).
+// Bound: a barrier (about 1.3 us) and one chain of dependent loads per phase.  As separate
+// launches a step of any mesh of up to 16k cells costs 46 us, 4.6 us for each of its ten
+// launches, whatever the size.
+// Each wait polls at most spin_limit times; one that gives up sets status bit 1 and its
+// block leaves (the others' waits then give up too).  The last block to leave clears the
+// barrier words for the next launch.
+struct StepsArgs {
+    StageArgs a;                 // common fields (status, scheme, flags)
+    double *u, *ust;             // FP64 state, and the stage value (FP64 path)
+    void *o0[3], *ord1, *ord2;   // order-0 records, order-1 and order-2 records
+    int n_diff, n_steps;
+    unsigned *bar;               // [0] arrivals, [32] blocks that left; zero between launches
+    unsigned spin_limit;
+};
+
+// Arrive and wait until all blocks have arrived `round` times; false if the wait gave up.
+__device__ __forceinline__ bool steps_barrier(const StepsArgs &q, unsigned round)
+{
+    __shared__ int ok;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        const unsigned target = round * gridDim.x;
+        asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(q.bar) : "memory");
+        unsigned it = 0, v;
+        for (;;) {
+            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(q.bar) : "memory");
+            if ((int)(v - target) >= 0 || ++it > q.spin_limit) break;
+        }
+        ok = it <= q.spin_limit;
+        if (!ok) atomicOr(q.a.status, 2u);
+    }
+    __syncthreads();
+    return ok;
+}
+
+template <int DIM, int NV, int PREC, int LPC>
+__global__ void __launch_bounds__(256) k_steps_small(DevMesh mesh, StepsArgs q)
+{
+    using R = typename PrecT<PREC>::R;
+    using T0 = typename PrecT<PREC>::T0;
+    constexpr int S0 = ord_stride<DIM, NV, 0, PREC>();
+    const int n = mesh.n_cells;
+    const long long tid = (long long)blockIdx.x * blockDim.x + threadIdx.x, nth = (long long)gridDim.x * blockDim.x;
+    const long long lanes = ((long long)n * LPC + 31) / 32 * 32;        // whole warps: they exchange by shuffles
+    unsigned round = 0;
+    bool ok = true;
+    for (long long c = tid; c < n; c += nth) {
+        R v[NV];
+#pragma unroll
+        for (int i = 0; i < NV; ++i) v[i] = (R)q.u[(long long)i * n + c];
+        store_rec<T0, NV, S0, R>(static_cast<T0 *>(q.o0[0]), c, v);
+    }
+    ok = steps_barrier(q, ++round);
+    StageArgs a = q.a;
+    a.ord[1] = q.ord1;
+    a.u0 = q.u;
+    a.rec_start = q.o0[0];
+    int cur = 0;
+    const int stages = 3 * q.n_steps;
+    for (int t = 0; ok && t < stages; ++t) {
+        const int sg = t % 3;
+        const bool last = t == stages - 1;
+        const int in = PREC == PREC_F64 ? cur : sg, nx = PREC == PREC_F64 ? 1 - cur : (sg == 2 ? 0 : sg + 1);
+        for (long long gt = tid; gt < lanes; gt += nth)
+            diff_cells<DIM, NV, 1, PREC, LPC, 0, false>(mesh, q.o0[in], q.ord1, gt, 0, 0, 0, nullptr);
+        if (!(ok = steps_barrier(q, ++round))) break;
+        a.ord[0] = q.o0[in];
+        a.o0_next = last ? nullptr : q.o0[nx];
+        if constexpr (PREC == PREC_F64) {
+            a.mode = 1;
+            a.us = sg == 0 ? q.u : q.ust;
+            a.out = sg < 2 ? q.ust : q.u;
+            a.A = sg == 0 ? 0.0 : sg == 1 ? 0.75 : 1.0 / 3.0;
+            a.B = sg == 0 ? 1.0 : sg == 1 ? 0.25 : 2.0 / 3.0;
+        } else {
+            a.mode = 2;
+            a.rk = sg;
+            a.out = q.u;
+        }
+        CoherentSrc<DIM, NV, PREC> src{a, mesh};
+        const long long work = q.n_diff >= 2 ? 2 * lanes : lanes;
+        for (long long gt = tid; gt < work; gt += nth) {
+            if (gt < lanes) stage_lanes<DIM, NV, 1, PREC, LPC>(mesh, a, src, gt);
+            else diff_cells<DIM, NV, 2, PREC, LPC, 0, false>(mesh, q.ord1, q.ord2, gt - lanes, 0, 0, 0, nullptr);
+        }
+        cur = 1 - cur;
+        if (!last) ok = steps_barrier(q, ++round);
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        if (atomicAdd(q.bar + 32, 1u) == gridDim.x - 1) {
+            q.bar[0] = 0;
+            q.bar[32] = 0;
+        }
     }
 }
 

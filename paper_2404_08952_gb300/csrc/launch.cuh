@@ -47,6 +47,9 @@ struct PathFns {
     void (*stage)(const DevMesh &, const StageArgs &, const Tune &, cudaStream_t);
     void (*faces)(const DevMesh &, const StageArgs &, double *, double *, cudaStream_t);
     void (*bnd_grad)(const DevMesh &, const void *, void *, cudaStream_t);
+    // whole steps in one cooperative launch with that many lanes per cell; null unless the
+    // stencil reads order 1 alone
+    cudaError_t (*steps_small)(const DevMesh &, const StepsArgs &, int lanes, cudaStream_t);
 };
 
 inline int nblk(long long n, int t) { return (int)((n + t - 1) / t); }
@@ -296,7 +299,32 @@ template <int DIM, int NV, int NS, int PREC> struct Path {
     {
         if (m.n_bcell > 0) k_bnd_grad<DIM, NV, PREC><<<nblk(m.n_bcell, 128), 128, 0, s>>>(m, o0, o1);
     }
-    static PathFns fns() { return PathFns{&pack, &diff, &diff_pair, &stage, &faces, &bnd_grad}; }
+    template <int LPC> static cudaError_t steps_l(const DevMesh &m, const StepsArgs &q, cudaStream_t s)
+    {
+        auto kern = k_steps_small<DIM, NV, PREC, LPC>;
+        constexpr int BS = 256;
+        const long long threads = ((long long)m.n_cells * LPC + 31) / 32 * 32 * (q.n_diff >= 2 ? 2 : 1);
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(std::min(nblk(threads, BS), persistent_grid((const void *)kern, BS, 0)));
+        cfg.blockDim = dim3(BS);
+        cfg.stream = s;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeCooperative;
+        attr[0].val.cooperative = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        return cudaLaunchKernelEx(&cfg, kern, m, q);
+    }
+    static cudaError_t steps_small(const DevMesh &m, const StepsArgs &q, int lanes, cudaStream_t s)
+    {
+        return lanes == 4 ? steps_l<4>(m, q, s) : steps_l<8>(m, q, s);
+    }
+    static PathFns fns()
+    {
+        PathFns f{&pack, &diff, &diff_pair, &stage, &faces, &bnd_grad, nullptr};
+        if constexpr (NS == 1) f.steps_small = &steps_small;
+        return f;
+    }
 };
 
 // Persistent batched stage (k_batch_stage), launched cooperatively.

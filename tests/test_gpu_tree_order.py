@@ -14,14 +14,14 @@ STENCIL = {2: (2, 1), 3: (3, 1), 4: (4, 1), 5: (5, 2)}
 
 def _mesh(name):
     if name == "tri":
-        return synth.tri_mesh(96, 91, jitter=0.2, seed=1)
+        return synth.tri_mesh(150, 137, jitter=0.2, seed=1)
     if name == "tri_open":
-        return synth.tri_mesh(101, 83, jitter=0.2, seed=2, boundary="transmissive")
+        return synth.tri_mesh(143, 145, jitter=0.2, seed=2, boundary="transmissive")
     if name == "tet":
-        return synth.tet_mesh((16, 14, 16), jitter=0.15, seed=3)
+        return synth.tet_mesh((20, 22, 20), jitter=0.15, seed=3)
     if name == "hexprism":
-        return synth.hexprism_mesh((23, 24, 25), jitter=0.2, seed=4)
-    return synth.hex_mesh(np.linspace(0, 1, 27), np.linspace(0, 1, 28), np.linspace(0, 1, 26) ** 1.3,
+        return synth.hexprism_mesh((31, 32, 33), jitter=0.2, seed=4)
+    return synth.hex_mesh(np.linspace(0, 1, 36), np.linspace(0, 1, 37), np.linspace(0, 1, 35) ** 1.3,
                           periodic=(True, True, False))
 
 
@@ -45,7 +45,7 @@ def test_untuned_shape_gives_the_lane_shape_bits(name, flux, order, n_diff, prec
     import torch
     m = _mesh(name)
     M = dg.Mesh(m)
-    assert M.n_cells >= 16384
+    assert M.n_cells >= 40000
     dim = M.dim
     nv = dim + 2 if flux == "rusanov" else 1
     k, r = STENCIL[order]
@@ -77,3 +77,56 @@ def test_untuned_shape_gives_the_lane_shape_bits(name, flux, order, n_diff, prec
     for a, b in zip(got, want):
         assert np.isfinite(a).all()
         np.testing.assert_array_equal(a, b)
+
+
+@pytest.mark.parametrize("name,args,flux,order,n_diff,precision,limiter", [
+    ("tri_mesh", (3, 4), "upwind", 3, 2, "fp64", "none"),
+    ("tri_mesh", (64, 64), "upwind", 3, 2, "fp64", "none"),
+    ("tri_mesh", (45, 37), "rusanov", 3, 2, "fp32", "first_order_flagged"),
+    ("tri_mesh", (37, 29), "burgers", 4, 2, "fp32_bf16", "none"),
+    ("tri_mesh", (150, 133), "rusanov", 2, 1, "fp32", "none"),
+    ("tet_mesh", ((4, 6, 4),), "rusanov", 3, 2, "fp32", "none"),
+    ("tet_mesh", ((20, 20, 18),), "rusanov", 3, 1, "fp64", "none"),
+    ("hexprism_mesh", ((5, 6, 7),), "upwind", 3, 2, "fp32", "none"),
+    ("hexprism_mesh", ((20, 21, 22),), "rusanov", 4, 2, "fp32_bf16", "none"),
+])
+def test_steps_of_a_small_mesh_in_one_launch(name, args, flux, order, n_diff, precision, limiter):
+    """Untuned steps of small meshes run in one cooperative launch: the bits of the separate
+    launches, also under stream capture, and a second call starts from clean barriers."""
+    import torch
+    m = getattr(synth, name)(*args, jitter=0.15, seed=7)
+    M = dg.Mesh(m)
+    assert M.n_cells <= 40000
+    dim = M.dim
+    nv = dim + 2 if flux == "rusanov" else 1
+    k, r = STENCIL[order]
+    sch = dg.Scheme(k=k, r=r, n_diff=n_diff, flux=flux, nv=nv, precision=precision, limiter=limiter,
+                    adv=(1.0, 0.7, -0.4)[:dim])
+    rng = np.random.default_rng(6)
+    s = 0.1 * rng.random(M.n_cells)
+    u0 = (1.0 + s)[None] if nv == 1 else np.stack([1.0 + s] + [0.4 + s] * dim + [3.0 + s])
+    flags = torch.from_numpy((rng.random(M.n_cells) < 0.3).astype(np.uint8)).cuda()
+    if limiter != "none":
+        dg.dolinc_set_flags(M, flags)
+    ws = dg.workspace(M, sch)
+    dt = 2e-3 / round(M.n_cells ** (1.0 / dim))
+    u = torch.from_numpy(u0).cuda()
+    dg.dolinc_rk_step(M, sch, dt, u, ws)
+    dg.dolinc_rk_steps(M, sch, dt, 3, u, ws)
+    got = u.cpu().numpy()
+    u.copy_(torch.from_numpy(u0))
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        dg.dolinc_rk_steps(M, sch, dt, 4, u, ws)
+    g.replay()
+    captured = u.cpu().numpy()
+    dg.dolinc_sync_status(M, ws)
+    lanes = 4 if name != "hexprism_mesh" else 8
+    dg.dolinc_set_tuning(M, sch, lanes, 256, lanes, 128)
+    u.copy_(torch.from_numpy(u0))
+    dg.dolinc_rk_steps(M, sch, dt, 4, u, ws)
+    want = u.cpu().numpy()
+    assert np.abs(want - u0).max() > 0
+    np.testing.assert_array_equal(got, want)
+    np.testing.assert_array_equal(captured, want)
