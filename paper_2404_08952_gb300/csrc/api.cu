@@ -360,8 +360,10 @@ constexpr int64_t kTreeCells = 40000;
 
 Tune tune_for(const dolinc_mesh *m, const dolinc_scheme *s)
 {
-    auto it = m->tuned.find(scheme_key(m, s));
-    if (it != m->tuned.end()) return it->second;
+    if (!m->tuned.empty()) {
+        auto it = m->tuned.find(scheme_key(m, s));
+        if (it != m->tuned.end()) return it->second;
+    }
     Tune t;
     const int lanes = m->max_faces <= 4 ? 4 : 8;
     t.diff_lpc = t.stage_lpc = lanes;             // one lane per face slot
@@ -793,11 +795,17 @@ namespace {
 // Whole steps of a small mesh in one launch (k_steps_small): untuned calls whose stencil
 // reads order 1 and that compute no order above 2, without Dirichlet/Neumann faces or
 // per-kernel timing.
-constexpr int64_t kSmallCells = 40000;
+// Measured per step, one launch against separate ones: 4k / 16k / 39k triangles FP32 Euler
+// 25 / 31 / 49 us against 54 / 50 / 54, 40k tetrahedra 65 against 67; FP64 advection on 8k /
+// 39k triangles 44 / 74 us against 58 / 81.  FP64 Euler needs twice the registers, so the
+// one resident grid holds fewer warps: 2.6k / 8.6k / 20k tetrahedra 77 / 107 / 182 us against
+// 92 / 141 / 167, 8k / 16k triangles 79 / 103 against 77 / 98.
+constexpr int64_t kSmallCells = 40000, kSmallCellsEuler64 = 8000;
 bool small_steps_ok(const dolinc_mesh *m, const PathFns *p, const dolinc_scheme *s)
 {
-    return p->steps_small && s->n_diff <= 2 && m->h.n_cells <= kSmallCells && m->max_faces <= 8 && m->d.n_bcell == 0 &&
-           !m->prof && !m->part && !m->tuned.count(scheme_key(m, s));
+    return p->steps_small && s->n_diff <= 2 && m->max_faces <= 8 &&
+           m->h.n_cells <= (s->precision == DOLINC_FP64 && s->nv > 1 ? kSmallCellsEuler64 : kSmallCells) &&
+           m->d.n_bcell == 0 && !m->prof && !m->part && (m->tuned.empty() || !m->tuned.count(scheme_key(m, s)));
 }
 
 cudaError_t small_steps(dolinc_mesh *m, const PathFns *p, const dolinc_scheme *s, double dt, double *u, void *ws,

@@ -1462,13 +1462,18 @@ __global__ void __launch_bounds__(256) k_batch_stage(DevMesh mesh, StageArgs a, 
 }
 
 // ------------------------------------------------------------------ persistent steps of small meshes
-// All stages of n_steps SSP-RK3 steps in one cooperative launch, LPC lanes per cell as
-// k_diff and k_stage run them (the same device code, so below FP64 the same bits).
-// Phases, separated by a grid barrier: pack | order 1 | stage and order 2 | order 1 | ..
-// (order 2 is read by nothing in the stage, so it runs beside it on other warps).
-// Bound: a barrier (about 1.3 us) and one chain of dependent loads per phase.  As separate
-// launches a step of any mesh of up to 16k cells costs 46 us, 4.6 us for each of its ten
-// launches, whatever the size.
+// All stages of n_steps SSP-RK3 steps in one cooperative launch.  Phases, separated by a
+// grid barrier: pack | order 1 | stage and order 2 | order 1 | .. (order 2 is read by
+// nothing in the stage, so it runs beside it on other threads).
+//   LPC 4, 8 (below FP64): lanes per cell as k_diff and k_stage run them, the same device
+//     code, so the same bits.  A phase is a barrier (about 1.3 us) and one chain of
+//     dependent loads, and lanes keep that chain short.
+//   LPC 0 (FP64): one thread per cell and the stage face-centric (every face once, then,
+//     after one more barrier, every cell's sum in slot order).  FP64 arithmetic bounds these
+//     meshes (two FMA per clock and SM), and lanes evaluate every face twice and issue for
+//     idle lanes: three times the FP64 instructions on triangles.
+// As separate launches a step of any mesh of up to 16k cells costs 46 us, 4.6 us for each
+// of its ten launches, whatever the size.
 // Each wait polls at most spin_limit times; one that gives up sets status bit 1 and its
 // block leaves (the others' waits then give up too).  The last block to leave clears the
 // barrier words for the next launch.
@@ -1501,24 +1506,27 @@ __device__ __forceinline__ bool steps_barrier(const StepsArgs &q, unsigned round
     return ok;
 }
 
+// Threads per block: 128 spread small FP64 meshes over the SMs (8192 triangles: 32 us a
+// step); with lanes 256 arrive at fewer barriers (16k triangles: 21 us a step, 128: 24).
+DOL_HD constexpr int steps_block(int lpc) { return lpc > 0 ? 256 : 128; }
+
 template <int DIM, int NV, int PREC, int LPC>
-__global__ void __launch_bounds__(256) k_steps_small(DevMesh mesh, StepsArgs q)
+__global__ void __launch_bounds__(steps_block(LPC)) k_steps_small(DevMesh mesh, StepsArgs q)
 {
     using R = typename PrecT<PREC>::R;
     using T0 = typename PrecT<PREC>::T0;
     constexpr int S0 = ord_stride<DIM, NV, 0, PREC>();
-    const int n = mesh.n_cells;
-    const long long tid = (long long)blockIdx.x * blockDim.x + threadIdx.x, nth = (long long)gridDim.x * blockDim.x;
-    const long long lanes = ((long long)n * LPC + 31) / 32 * 32;        // whole warps: they exchange by shuffles
+    const int n = mesh.n_cells, nf = mesh.n_faces;
+    const int tid = blockIdx.x * steps_block(LPC) + threadIdx.x, nth = gridDim.x * steps_block(LPC);
+    const int lanes = LPC > 0 ? (n * LPC + 31) / 32 * 32 : n;           // whole warps: they exchange by shuffles
     unsigned round = 0;
-    bool ok = true;
-    for (long long c = tid; c < n; c += nth) {
+    for (int c = tid; c < n; c += nth) {
         R v[NV];
 #pragma unroll
         for (int i = 0; i < NV; ++i) v[i] = (R)q.u[(long long)i * n + c];
         store_rec<T0, NV, S0, R>(static_cast<T0 *>(q.o0[0]), c, v);
     }
-    ok = steps_barrier(q, ++round);
+    bool ok = steps_barrier(q, ++round);
     StageArgs a = q.a;
     a.ord[1] = q.ord1;
     a.u0 = q.u;
@@ -1529,8 +1537,10 @@ __global__ void __launch_bounds__(256) k_steps_small(DevMesh mesh, StepsArgs q)
         const int sg = t % 3;
         const bool last = t == stages - 1;
         const int in = PREC == PREC_F64 ? cur : sg, nx = PREC == PREC_F64 ? 1 - cur : (sg == 2 ? 0 : sg + 1);
-        for (long long gt = tid; gt < lanes; gt += nth)
-            diff_cells<DIM, NV, 1, PREC, LPC, 0, false>(mesh, q.o0[in], q.ord1, gt, 0, 0, 0, nullptr);
+        for (int i = tid; i < lanes; i += nth) {
+            if constexpr (LPC > 0) diff_cells<DIM, NV, 1, PREC, LPC, 0, false>(mesh, q.o0[in], q.ord1, i, 0, 0, 0, nullptr);
+            else diff_cell<DIM, NV, 1, PREC>(mesh, q.o0[in], q.ord1, i);
+        }
         if (!(ok = steps_barrier(q, ++round))) break;
         a.ord[0] = q.o0[in];
         a.o0_next = last ? nullptr : q.o0[nx];
@@ -1546,10 +1556,41 @@ __global__ void __launch_bounds__(256) k_steps_small(DevMesh mesh, StepsArgs q)
             a.out = q.u;
         }
         CoherentSrc<DIM, NV, PREC> src{a, mesh};
-        const long long work = q.n_diff >= 2 ? 2 * lanes : lanes;
-        for (long long gt = tid; gt < work; gt += nth) {
-            if (gt < lanes) stage_lanes<DIM, NV, 1, PREC, LPC>(mesh, a, src, gt);
-            else diff_cells<DIM, NV, 2, PREC, LPC, 0, false>(mesh, q.ord1, q.ord2, gt - lanes, 0, 0, 0, nullptr);
+        const int first = LPC > 0 ? lanes : nf, work = first + (q.n_diff >= 2 ? lanes : 0);
+        for (int i = tid; i < work; i += nth) {
+            if constexpr (LPC > 0) {
+                if (i < first) stage_lanes<DIM, NV, 1, PREC, LPC>(mesh, a, src, i);
+                else diff_cells<DIM, NV, 2, PREC, LPC, 0, false>(mesh, q.ord1, q.ord2, i - first, 0, 0, 0, nullptr);
+            } else if (i < first) {
+                const int P = __ldg(mesh.fo + i), N = __ldg(mesh.fn + i);
+                R F[NV];
+                canon_flux<DIM, NV, 1, PREC>(a, src, P, N < 0 ? P : N, ((unsigned)i << 2) | (N < 0 ? 2u : 0u),
+                                             a.flags && a.flags[P], F);
+#pragma unroll
+                for (int v = 0; v < NV; ++v) static_cast<R *>(a.face_flux)[(long long)v * nf + i] = F[v];
+            } else {
+                diff_cell<DIM, NV, 2, PREC>(mesh, q.ord1, q.ord2, i - first);
+            }
+        }
+        if constexpr (LPC == 0) {
+            if (!(ok = steps_barrier(q, ++round))) break;
+            for (int c = tid; c < n; c += nth) {
+                const R *flux = static_cast<const R *>(a.face_flux);
+                R res[NV];
+#pragma unroll
+                for (int v = 0; v < NV; ++v) res[v] = (R)0;
+                int s0, s1;
+                slot_range(mesh, c, s0, s1);
+                for (int s = s0; s < s1; ++s) {
+                    const unsigned word = __ldg(mesh.sword + s);
+#pragma unroll
+                    for (int v = 0; v < NV; ++v) {
+                        const R F = flux[(long long)v * nf + (word >> 2)];
+                        res[v] += (word & 1) ? F : -F;
+                    }
+                }
+                cell_epilogue<DIM, NV, PREC>(mesh, a, c, res);
+            }
         }
         cur = 1 - cur;
         if (!last) ok = steps_barrier(q, ++round);

@@ -302,8 +302,9 @@ template <int DIM, int NV, int NS, int PREC> struct Path {
     template <int LPC> static cudaError_t steps_l(const DevMesh &m, const StepsArgs &q, cudaStream_t s)
     {
         auto kern = k_steps_small<DIM, NV, PREC, LPC>;
-        constexpr int BS = 256;
-        const long long threads = ((long long)m.n_cells * LPC + 31) / 32 * 32 * (q.n_diff >= 2 ? 2 : 1);
+        constexpr int BS = steps_block(LPC);
+        const long long first = LPC > 0 ? ((long long)m.n_cells * LPC + 31) / 32 * 32 : m.n_faces;
+        const long long threads = first + (q.n_diff < 2 ? 0 : LPC > 0 ? first : m.n_cells);
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(std::min(nblk(threads, BS), persistent_grid((const void *)kern, BS, 0)));
         cfg.blockDim = dim3(BS);
@@ -317,7 +318,8 @@ template <int DIM, int NV, int NS, int PREC> struct Path {
     }
     static cudaError_t steps_small(const DevMesh &m, const StepsArgs &q, int lanes, cudaStream_t s)
     {
-        return lanes == 4 ? steps_l<4>(m, q, s) : steps_l<8>(m, q, s);
+        if constexpr (PREC == PREC_F64) return steps_l<0>(m, q, s);
+        else return lanes == 4 ? steps_l<4>(m, q, s) : steps_l<8>(m, q, s);
     }
     static PathFns fns()
     {

@@ -86,7 +86,8 @@ def test_untuned_shape_gives_the_lane_shape_bits(name, flux, order, n_diff, prec
     ("tri_mesh", (37, 29), "burgers", 4, 2, "fp32_bf16", "none"),
     ("tri_mesh", (150, 133), "rusanov", 2, 1, "fp32", "none"),
     ("tet_mesh", ((4, 6, 4),), "rusanov", 3, 2, "fp32", "none"),
-    ("tet_mesh", ((20, 20, 18),), "rusanov", 3, 1, "fp64", "none"),
+    ("tet_mesh", ((12, 10, 12),), "rusanov", 3, 1, "fp64", "none"),
+    ("hexprism_mesh", ((20, 21, 22),), "upwind", 4, 2, "fp64", "none"),
     ("hexprism_mesh", ((5, 6, 7),), "upwind", 3, 2, "fp32", "none"),
     ("hexprism_mesh", ((20, 21, 22),), "rusanov", 4, 2, "fp32_bf16", "none"),
 ])
@@ -123,7 +124,7 @@ def test_steps_of_a_small_mesh_in_one_launch(name, args, flux, order, n_diff, pr
     captured = u.cpu().numpy()
     dg.dolinc_sync_status(M, ws)
     lanes = 4 if name != "hexprism_mesh" else 8
-    dg.dolinc_set_tuning(M, sch, lanes, 256, lanes, 128)
+    dg.dolinc_set_tuning(M, sch, *((1, 64, -2, 64) if precision == "fp64" else (lanes, 256, lanes, 128)))
     u.copy_(torch.from_numpy(u0))
     dg.dolinc_rk_steps(M, sch, dt, 4, u, ws)
     want = u.cpu().numpy()
