@@ -2232,6 +2232,8 @@ dolinc_status dolinc_implicit_step(dolinc_implicit *imp, double *u, int n_outer,
     a.tol2 = imp->rel_tol * imp->rel_tol;
     a.max_iter = imp->max_iter;
     a.spin_limit = imp->spin_limit;
+    a.uniform = m->d.uniform_slots;
+    const bool in_sm = imp->ell == 0 && imp->n <= imp_sm_cells(imp->sms);
     for (int k = 0; k < n_outer; ++k) {
         double *Rk = k == 0 ? imp->Rn : imp->R;
         dolinc_status st = dolinc_residual(m, &imp->s, u, Rk, ws, ws_bytes, stream);
@@ -2248,7 +2250,9 @@ dolinc_status dolinc_implicit_step(dolinc_implicit *imp, double *u, int n_outer,
         a.x2 = imp->xw[(imp->xw_last + 2) % 3];
         a.x = first ? imp->xw[(imp->xw_last + 1) % 3] : imp->vec[0];
         cudaError_t e = cudaSuccess;
-        timed(m, DOLINC_KERNEL_SOLVE, cs, [&] { e = launch_imp_solve(a, imp->ell, imp->grid, cs); });
+        timed(m, DOLINC_KERNEL_SOLVE, cs, [&] {
+            e = in_sm ? launch_imp_solve_sm(a, imp->sms, cs) : launch_imp_solve(a, imp->ell, imp->grid, cs);
+        });
         if (e != cudaSuccess) {
             cudaGetLastError();
             return fail(DOLINC_ERR_CUDA, std::string("cooperative launch: ") + cudaGetErrorString(e));

@@ -40,6 +40,7 @@ struct ImpSolve {
     const double *x1, *x2;       // the previous steps' solutions (warm >= 1, warm = 2)
     int max_iter;
     unsigned spin_limit;
+    int uniform;                 // slots of every cell when all have the same number, else 0
 };
 
 // Layout of ImpSolve::scal.  Iteration counts accumulate over the solves of a step;
@@ -50,6 +51,11 @@ enum { SC_RHO = 0, SC_ALPHA, SC_OMEGA, SC_BETA, SC_BB, SC_RR, SC_DONE, SC_ITERS,
 int imp_ell_width(int max_slots);
 cudaError_t launch_imp_solve(const ImpSolve &a, int ell, int grid, cudaStream_t s);
 int imp_solve_blocks_per_sm(int ell);
+// rows per slot and at most imp_sm_cells cells: the solve with a chunk of cells per SM in
+// shared memory (bar: [32] blocks that left, [64] abort; life[2]: the tag its posts go
+// on from; part: 2 sets of IMP_NRED 16-byte words per SM)
+int64_t imp_sm_cells(int sms);
+cudaError_t launch_imp_solve_sm(const ImpSolve &a, int sms, cudaStream_t s);
 constexpr int IMP_BLOCK = 256;
 constexpr int IMP_NRED = 4;      // values a grid barrier reduces at most (partials per block)
 
