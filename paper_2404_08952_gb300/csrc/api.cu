@@ -307,7 +307,11 @@ StageArgs base_args(const dolinc_mesh *m, const dolinc_scheme *s, void *ws, cons
     a.r = s->r;
     a.flux = s->flux;
     a.gamma = s->gamma;
-    for (int i = 0; i < 3; ++i) a.adv[i] = s->adv[i];
+    a.gamma32 = (float)s->gamma;
+    for (int i = 0; i < 3; ++i) {
+        a.adv[i] = s->adv[i];
+        a.adv32[i] = (float)s->adv[i];
+    }
     const bool flagged = s->limiter == DOLINC_LIMIT_ENO3_FLAGGED || s->limiter == DOLINC_LIMIT_FIRST_ORDER_FLAGGED ||
                          s->limiter == DOLINC_LIMIT_WENO5_FLAGGED;
     a.flags = flagged ? m->flags : nullptr;
@@ -317,6 +321,12 @@ StageArgs base_args(const dolinc_mesh *m, const dolinc_scheme *s, void *ws, cons
                                                                  : LIM_ENO3;
     a.face_flux = B(ws, L.flux);
     return a;
+}
+
+void set_dt(StageArgs &a, double dt)
+{
+    a.dt = dt;
+    a.dt32 = (float)dt;
 }
 
 cudaEvent_t take_event(dolinc_mesh *m)
@@ -782,7 +792,7 @@ dolinc_status dolinc_rk_stage(dolinc_mesh *m, const dolinc_scheme *s, double dt,
     a.out = out;
     a.A = A[stage];
     a.B = Bc[stage];
-    a.dt = dt;
+    set_dt(a, dt);
     a.o0_next = nullptr;
     timed(m, DOLINC_KERNEL_STAGE, cs, [&] { p->stage(m->d, a, tune_for(m, s), cs); });
     return launch_check();
@@ -813,7 +823,7 @@ cudaError_t small_steps(dolinc_mesh *m, const PathFns *p, const dolinc_scheme *s
 {
     StepsArgs q{};
     q.a = base_args(m, s, ws, L, L.o0[0]);
-    q.a.dt = dt;
+    set_dt(q.a, dt);
     q.a.dacc = reinterpret_cast<float *>(B(ws, L.dacc));
     q.u = u;
     q.ust = reinterpret_cast<double *>(B(ws, L.ustage));
@@ -896,7 +906,7 @@ dolinc_status rk_step_impl(dolinc_mesh *m, const dolinc_scheme *s, double dt, co
                 a.rk = sg;
                 a.u0 = u_dev;
                 a.out = last ? u_out : u_dev;
-                a.dt = dt;
+                set_dt(a, dt);
                 a.dacc = reinterpret_cast<float *>(B(ws, L.dacc));
                 a.rec_start = B(ws, L.o0[0]);
                 a.o0_next = sg < 2 ? B(ws, L.o0[sg + 1]) : (last ? nullptr : B(ws, L.o0[0]));
@@ -923,7 +933,7 @@ dolinc_status rk_step_impl(dolinc_mesh *m, const dolinc_scheme *s, double dt, co
             a.out = sg < 2 ? ust : (last ? u_out : u_dev);
             a.A = A[sg];
             a.B = Bc[sg];
-            a.dt = dt;
+            set_dt(a, dt);
             a.o0_next = (sg == 2 && last) ? nullptr : B(ws, L.o0[1 - cur]);
             timed(m, DOLINC_KERNEL_STAGE, cs, [&] { p->stage(m->d, a, tn, cs); });
             cur = 1 - cur;
@@ -1096,7 +1106,7 @@ dolinc_status dolinc_autotune(dolinc_mesh *m, const dolinc_scheme *s, const doub
                 StageArgs a = base_args(m, s, ws, L, L.o0[0]);
                 double *scratch = reinterpret_cast<double *>(B(ws, L.ustage));
                 a.u0 = a.us = a.out = scratch;
-                a.dt = 0.0;
+                set_dt(a, 0.0);
                 if (s->precision != DOLINC_FP64) {
                     a.mode = 2;
                     a.rk = 1;
@@ -1771,7 +1781,7 @@ dolinc_status part_advance(dolinc_mesh *m, const dolinc_scheme *s, void *ws, con
     // every order the stage reads is in place on the ghosts: the stage kernel
     const int sg = P.stage;
     StageArgs a = base_args(m, s, ws, L, o0off);
-    a.dt = P.dt;
+    set_dt(a, P.dt);
     a.u0 = P.u;
     if (s->precision != DOLINC_FP64) {
         a.mode = 2;

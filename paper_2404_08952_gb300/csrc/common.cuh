@@ -57,6 +57,34 @@ template <> __device__ __forceinline__ float sqrt_bulk<float>(float x)
 template <> __device__ __forceinline__ __nv_bfloat16 to_store<__nv_bfloat16, float>(float x) { return __float2bfloat16_rn(x); }
 template <> __device__ __forceinline__ __nv_bfloat16 to_store<__nv_bfloat16, double>(double x) { return __float2bfloat16_rn((float)x); }
 
+// FP64 <-> bulk precision.  The chip converts between 32 and 64 bits on the FP64 pipe, two
+// threads per clock and SM (the last stage's gather of 5 variables on 1.31M cells: 31 us of
+// that pipe for two conversions and an add each), so values in the normal range are
+// converted by integer operations, with the same result: round to nearest even.  Zeros too;
+// the rest (subnormal results, overflow, infinities, NaN) takes the instruction.
+template <class R> __device__ __forceinline__ R narrow(double x) { return (R)x; }
+template <> __device__ __forceinline__ float narrow<float>(double x)
+{
+    const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+    const unsigned sign = hi & 0x80000000u, e = (hi >> 20) & 0x7ffu;
+    if (e - 897u < 253u) {                           // float exponent 1..253: a carry stays normal
+        unsigned f = ((hi & 0x7fffffffu) << 3 | lo >> 29) - (896u << 23);
+        f += ((lo << 3) | (f & 1u)) > 0x80000000u;
+        return __uint_as_float(sign | f);
+    }
+    if (((hi << 1) | lo) == 0u) return __uint_as_float(sign);
+    return (float)x;
+}
+__device__ __forceinline__ double widen(double x) { return x; }
+__device__ __forceinline__ double widen(float x)
+{
+    const unsigned b = __float_as_uint(x), a = b & 0x7fffffffu;
+    if ((b >> 23 & 0xffu) - 1u < 254u)
+        return __hiloint2double((int)((b & 0x80000000u) | ((a >> 3) + (896u << 20))), (int)(b << 29));
+    if (a == 0u) return __hiloint2double((int)b, 0);
+    return (double)x;
+}
+
 // ------------------------------------------------------------------ record load/store
 // Loads the first N elements of a record of stride S (elements of T) into registers.
 // LDG: read through the read-only data path (global memory only); otherwise a generic

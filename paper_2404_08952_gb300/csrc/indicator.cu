@@ -85,7 +85,7 @@ __global__ void __launch_bounds__(128) k_criterion(DevMesh mesh, StageArgs a, fl
             }
             UR[v] = t;
         }
-        const R gam = (R)a.gamma;
+        const R gam = par_gamma<R>(a);
         if (!(UL[0] > (R)0) || !(pressure_of<DIM, R>(gam, UL) > (R)0) || !(UR[0] > (R)0) ||
             !(pressure_of<DIM, R>(gam, UR) > (R)0))
             trouble = true;
@@ -175,6 +175,17 @@ __device__ __forceinline__ bool lex_gt(const float *a, const float *b)
     return false;
 }
 
+// the 6 features of cell c (24-byte records)
+__device__ __forceinline__ void load6(const float *__restrict__ own, int c, float *f)
+{
+    const float2 *p = reinterpret_cast<const float2 *>(own + 6ll * c);
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+        const float2 v = __ldg(p + q);
+        f[2 * q] = v.x, f[2 * q + 1] = v.y;
+    }
+}
+
 // Network input of cell c: its own 6 features, then the 6 of the three largest face
 // neighbours in lexicographic order (itself across a boundary face).
 __device__ __forceinline__ void gather24_cell(const DevMesh &mesh, const float *__restrict__ own, int c, float *o)
@@ -186,8 +197,7 @@ __device__ __forceinline__ void gather24_cell(const DevMesh &mesh, const float *
     for (int s = s0; s < s1; ++s) {
         const int nb = __ldg(mesh.slot2 + s).x;
         float f[6];
-#pragma unroll
-        for (int q = 0; q < 6; ++q) f[q] = __ldg(own + 6ll * nb + q);
+        load6(own, nb, f);
         // insert into the descending top-3 list (compile-time indices only)
         bool ins0 = have < 1 || lex_gt(f, top[0]);
         bool ins1 = !ins0 && (have < 2 || lex_gt(f, top[1]));
@@ -202,8 +212,7 @@ __device__ __forceinline__ void gather24_cell(const DevMesh &mesh, const float *
         if (have < 3) ++have;
     }
     float self[6];
-#pragma unroll
-    for (int q = 0; q < 6; ++q) self[q] = __ldg(own + 6ll * c + q);
+    load6(own, c, self);
 #pragma unroll
     for (int a = 0; a < 3; ++a)
         if (a >= have)
@@ -261,17 +270,24 @@ __device__ __forceinline__ void mma_bf16(float *d, const uint32_t *a, uint2 b)
                  : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b.x), "r"(b.y));
 }
 
-// 16 cells per warp tile; activations stay in registers between layers (the f32
-// accumulator layout of two adjacent n-tiles is the bf16 A layout of one k-tile).
-// FUSED: the inputs are not read from x but gathered per tile (gather24_cell, lanes
-// 0-15 one cell each) into the warp's 16 x 24 shared-memory rows.
+// 32 cells per warp tile, two m16 tiles that share every B fragment read from shared
+// memory (with 16 cells the fragments' reads, 84 of 256 bytes per tile, were the kernel's
+// largest cost).  Activations stay in registers between layers (the f32 accumulator layout
+// of two adjacent n-tiles is the bf16 A layout of one k-tile).
+// The tile's inputs are staged as bf16 pairs, 12 words per cell (rows of 12 words put the
+// 32 words of an A fragment in distinct banks).  FUSED: they are not read from x but
+// gathered (gather24_cell, one cell per lane).
+// Bound: the tensor pipe and the shared-memory reads.  1.05M triangles, fused: see the
+// table in the design notes for the time; 16 cells per tile took 121 us.
+constexpr int XW = MLP_IN / 2;
+
 template <bool FUSED>
-__global__ void __launch_bounds__(128) k_mlp_infer(const uint2 *__restrict__ frag, const float *__restrict__ theta,
+__global__ void __launch_bounds__(128, 4) k_mlp_infer(const uint2 *__restrict__ frag, const float *__restrict__ theta,
                                                    const float *__restrict__ x, long long n,
                                                    float *__restrict__ logits, uint8_t *__restrict__ flags,
                                                    DevMesh mesh, const float *__restrict__ own)
 {
-    __shared__ float sx[FUSED ? 4 * 16 * MLP_IN : 1];
+    __shared__ uint32_t sx[4][32][XW];
     __shared__ uint2 sfrag[N_FRAGS * 32];
     __shared__ float sbias[3 * MLP_H + 1];
     for (int i = threadIdx.x; i < N_FRAGS * 32; i += blockDim.x) sfrag[i] = frag[i];
@@ -285,63 +301,87 @@ __global__ void __launch_bounds__(128) k_mlp_infer(const uint2 *__restrict__ fra
     const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
     const long long warps = (long long)gridDim.x * (blockDim.x / 32);
     const long long w0 = (long long)blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
-    for (long long tile = w0; tile * 16 < n; tile += warps) {
-        const long long r0 = tile * 16 + g, r1 = r0 + 8;
-        float *wx = sx + (FUSED ? (threadIdx.x / 32) * 16 * MLP_IN : 0);
+    uint32_t (*wx)[XW] = sx[threadIdx.x / 32];
+    for (long long tile = w0; tile * 32 < n; tile += warps) {
+        const long long c0 = tile * 32;
+        __syncwarp();
         if constexpr (FUSED) {
-            __syncwarp();
-            const long long cr = tile * 16 + lane;
-            if (lane < 16 && cr < n) gather24_cell(mesh, own, (int)cr, wx + lane * MLP_IN);
-            __syncwarp();
-        }
-        // layer 1 input: 24 features padded to 32 (two k-tiles)
-        uint32_t A[4][4];
-        auto xv = [&](long long r, int col) {
-            if (r >= n || col >= MLP_IN) return 0.0f;
-            if constexpr (FUSED) return wx[(r - tile * 16) * MLP_IN + col];
-            else return __ldg(x + r * MLP_IN + col);
-        };
+            if (c0 + lane < n) {
+                float o[MLP_IN];
+                gather24_cell(mesh, own, (int)(c0 + lane), o);
 #pragma unroll
-        for (int kt = 0; kt < 2; ++kt) {
-            const int c0 = 16 * kt + 2 * t;
-            A[kt][0] = pack_bf16(xv(r0, c0), xv(r0, c0 + 1));
-            A[kt][1] = pack_bf16(xv(r1, c0), xv(r1, c0 + 1));
-            A[kt][2] = pack_bf16(xv(r0, c0 + 8), xv(r0, c0 + 9));
-            A[kt][3] = pack_bf16(xv(r1, c0 + 8), xv(r1, c0 + 9));
+                for (int q = 0; q < XW; ++q) wx[lane][q] = pack_bf16(o[2 * q], o[2 * q + 1]);
+            }
+        } else {
+            // the tile's rows are contiguous: 16-byte pieces where the tile is whole and x
+            // is aligned to them, else single values
+            const float *xt = x + c0 * MLP_IN;
+            if (c0 + 32 <= n && (reinterpret_cast<uintptr_t>(x) & 15) == 0) {
+#pragma unroll
+                for (int q = 0; q < MLP_IN / 4; ++q) {
+                    const int i = lane + 32 * q;
+                    const float4 v = __ldg(reinterpret_cast<const float4 *>(xt) + i);
+                    (&wx[0][0])[2 * i] = pack_bf16(v.x, v.y);
+                    (&wx[0][0])[2 * i + 1] = pack_bf16(v.z, v.w);
+                }
+            } else {
+                for (int i = lane; i < 32 * XW; i += 32)
+                    if (c0 + i / XW < n) (&wx[0][0])[i] = pack_bf16(__ldg(xt + 2 * i), __ldg(xt + 2 * i + 1));
+            }
         }
-        float C[8][4];
+        __syncwarp();
+        // layer 1 input: 24 features padded to 32 (two k-tiles); rows past n are not stored
+        uint32_t A[2][4][4];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const uint32_t *p0 = wx[16 * h + g], *p1 = wx[16 * h + g + 8];
+            A[h][0][0] = p0[t], A[h][0][1] = p1[t], A[h][0][2] = p0[t + 4], A[h][0][3] = p1[t + 4];
+            A[h][1][0] = p0[t + 8], A[h][1][1] = p1[t + 8], A[h][1][2] = A[h][1][3] = 0u;
+        }
         // three hidden layers
 #pragma unroll
         for (int layer = 0; layer < 3; ++layer) {
             const int nk = layer == 0 ? 2 : 4;
             const int fbase = layer == 0 ? FRAG_L1 : (layer == 1 ? FRAG_L2 : FRAG_L3);
+            float C[2][8][4];
 #pragma unroll
             for (int nt = 0; nt < 8; ++nt) {
                 const float b0 = sbias[layer * MLP_H + 8 * nt + 2 * t], b1 = sbias[layer * MLP_H + 8 * nt + 2 * t + 1];
-                C[nt][0] = b0; C[nt][1] = b1; C[nt][2] = b0; C[nt][3] = b1;
+#pragma unroll
+                for (int h = 0; h < 2; ++h) C[h][nt][0] = b0, C[h][nt][1] = b1, C[h][nt][2] = b0, C[h][nt][3] = b1;
 #pragma unroll
                 for (int kt = 0; kt < 4; ++kt)
-                    if (kt < nk) mma_bf16(C[nt], A[kt], sfrag[(fbase + kt * 8 + nt) * 32 + lane]);
+                    if (kt < nk) {
+                        const uint2 B = sfrag[(fbase + kt * 8 + nt) * 32 + lane];
+                        mma_bf16(C[0][nt], A[0][kt], B);
+                        mma_bf16(C[1][nt], A[1][kt], B);
+                    }
             }
 #pragma unroll
-            for (int kt = 0; kt < 4; ++kt) {
-                A[kt][0] = pack_bf16(fmaxf(C[2 * kt][0], 0.f), fmaxf(C[2 * kt][1], 0.f));
-                A[kt][1] = pack_bf16(fmaxf(C[2 * kt][2], 0.f), fmaxf(C[2 * kt][3], 0.f));
-                A[kt][2] = pack_bf16(fmaxf(C[2 * kt + 1][0], 0.f), fmaxf(C[2 * kt + 1][1], 0.f));
-                A[kt][3] = pack_bf16(fmaxf(C[2 * kt + 1][2], 0.f), fmaxf(C[2 * kt + 1][3], 0.f));
-            }
+            for (int h = 0; h < 2; ++h)
+#pragma unroll
+                for (int kt = 0; kt < 4; ++kt) {
+                    A[h][kt][0] = pack_bf16(fmaxf(C[h][2 * kt][0], 0.f), fmaxf(C[h][2 * kt][1], 0.f));
+                    A[h][kt][1] = pack_bf16(fmaxf(C[h][2 * kt][2], 0.f), fmaxf(C[h][2 * kt][3], 0.f));
+                    A[h][kt][2] = pack_bf16(fmaxf(C[h][2 * kt + 1][0], 0.f), fmaxf(C[h][2 * kt + 1][1], 0.f));
+                    A[h][kt][3] = pack_bf16(fmaxf(C[h][2 * kt + 1][2], 0.f), fmaxf(C[h][2 * kt + 1][3], 0.f));
+                }
         }
-        float O[4] = {sbias[3 * MLP_H], 0.f, sbias[3 * MLP_H], 0.f};
 #pragma unroll
-        for (int kt = 0; kt < 4; ++kt) mma_bf16(O, A[kt], sfrag[(FRAG_L4 + kt) * 32 + lane]);
-        if (t == 0) {
-            if (r0 < n) {
-                if (logits) logits[r0] = O[0];
-                if (flags) flags[r0] = O[0] > 0.f;
-            }
-            if (r1 < n) {
-                if (logits) logits[r1] = O[2];
-                if (flags) flags[r1] = O[2] > 0.f;
+        for (int h = 0; h < 2; ++h) {
+            float O[4] = {sbias[3 * MLP_H], 0.f, sbias[3 * MLP_H], 0.f};
+#pragma unroll
+            for (int kt = 0; kt < 4; ++kt) mma_bf16(O, A[h][kt], sfrag[(FRAG_L4 + kt) * 32 + lane]);
+            const long long r0 = c0 + 16 * h + g, r1 = r0 + 8;
+            if (t == 0) {
+                if (r0 < n) {
+                    if (logits) logits[r0] = O[0];
+                    if (flags) flags[r0] = O[0] > 0.f;
+                }
+                if (r1 < n) {
+                    if (logits) logits[r1] = O[2];
+                    if (flags) flags[r1] = O[2] > 0.f;
+                }
             }
         }
     }
@@ -641,9 +681,9 @@ void launch_mlp_frags(const float *theta, uint2 *frag, cudaStream_t s)
 void launch_mlp_infer(const uint2 *frag, const float *theta, const float *x, long long n, float *logits,
                       uint8_t *flags, cudaStream_t s)
 {
-    long long tiles = (n + 15) / 16;
+    long long tiles = (n + 31) / 32;
     int blocks = (int)((tiles + 3) / 4);
-    if (blocks > 152 * 16) blocks = 152 * 16;
+    if (blocks > 152 * 8) blocks = 152 * 8;
     if (blocks < 1) blocks = 1;
     k_mlp_infer<false><<<blocks, 128, 0, s>>>(frag, theta, x, n, logits, flags, DevMesh{}, nullptr);
 }
@@ -651,9 +691,9 @@ void launch_mlp_infer_fused(const uint2 *frag, const float *theta, const DevMesh
                             uint8_t *flags, cudaStream_t s)
 {
     const long long n = m.n_cells;
-    long long tiles = (n + 15) / 16;
+    long long tiles = (n + 31) / 32;
     int blocks = (int)((tiles + 3) / 4);
-    if (blocks > 152 * 16) blocks = 152 * 16;
+    if (blocks > 152 * 8) blocks = 152 * 8;
     if (blocks < 1) blocks = 1;
     k_mlp_infer<true><<<blocks, 128, 0, s>>>(frag, theta, nullptr, n, logits, flags, m, own);
 }
