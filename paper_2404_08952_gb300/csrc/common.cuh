@@ -304,38 +304,12 @@ __device__ __forceinline__ void monomials(R dx, R dy, R dz, R *mono)
 // the primitive at the stencil's faces (face x_{i+1/2} = 0 is node r+1).
 // Step 2: the transpose of the far-field recursion moves each far cell's weight onto
 // the two face cells' differentials.
-template <int NS, class R>
-__device__ __forceinline__ void dolinc_weights(int k, int r, R g, R *W0, R *W1)
+// The general stencil.  KC, RC > 0: (k, r) known at compile time, the same operations
+// without a select for each candidate position.
+template <int NS, class R, int KC, int RC>
+__device__ __forceinline__ void dolinc_weights_general(int k_, int r_, R g, R *W0, R *W1)
 {
-    if (r == 1 && k >= 2 && k <= 4) {
-        // First-order DOLINC stencils in closed form (Sec 2.4: Eq coeff on geometric
-        // cells combined with Eqs lCoeffDLC1/rCoeffDLC1), G_n = 1 + g + .. + g^(n-1):
-        //  (2,1):      W0 = ((2+g), 1)/G2,                       W1 = (-1, 0)/G2
-        //  (3,1) USR3: W0 = (g(1+3g+g^2), g^2)/(G2 G3),          W1 = (1+g-g^2, 0)/(G2 G3)
-        //  (4,1) CSR4: W0 = (-g+g^2+2g^3+3g^4+g^5, g^4)/(G3 G4), W1 = (1+3g+2g^2+g^3-g^4, -g)/(G3 G4)
-        const R g2 = g * g;
-#pragma unroll
-        for (int m = 0; m <= NS; ++m) W0[m] = W1[m] = (R)0;
-        if (k == 2) {
-            const R iv = rcp_bulk((R)1 + g);
-            W0[0] = ((R)2 + g) * iv;
-            W0[1] = iv;
-            W1[0] = -iv;
-        } else if (k == 3) {
-            const R iv = rcp_bulk(((R)1 + g) * ((R)1 + g + g2));
-            W0[0] = g * ((R)1 + (R)3 * g + g2) * iv;
-            W0[1] = g2 * iv;
-            W1[0] = ((R)1 + g - g2) * iv;
-        } else {
-            const R g3 = g2 * g, g4 = g2 * g2;
-            const R iv = rcp_bulk(((R)1 + g + g2) * ((R)1 + g + g2 + g3));
-            W0[0] = (-g + g2 + (R)2 * g3 + (R)3 * g4 + g4 * g) * iv;
-            W0[1] = g4 * iv;
-            W1[0] = ((R)1 + (R)3 * g + (R)2 * g2 + g3 - g4) * iv;
-            W1[1] = -g * iv;
-        }
-        return;
-    }
+    const int k = KC > 0 ? KC : k_, r = KC > 0 ? RC : r_;
     constexpr int KM = 2 * NS + 2;
     R gi = (R)1 / g;
     // face positions x_q = right face of cell i-r+q-1, q = 0..k
@@ -435,6 +409,45 @@ __device__ __forceinline__ void dolinc_weights(int k, int r, R g, R *W0, R *W1)
     }
 #pragma unroll
     for (int m = 0; m <= NS; ++m) { W0[m] = wt[NS][m]; W1[m] = wt[NS + 1][m]; }
+}
+
+template <int NS, class R>
+__device__ __forceinline__ void dolinc_weights(int k, int r, R g, R *W0, R *W1)
+{
+    if (r == 1 && k >= 2 && k <= 4) {
+        // First-order DOLINC stencils in closed form (Sec 2.4: Eq coeff on geometric
+        // cells combined with Eqs lCoeffDLC1/rCoeffDLC1), G_n = 1 + g + .. + g^(n-1):
+        //  (2,1):      W0 = ((2+g), 1)/G2,                       W1 = (-1, 0)/G2
+        //  (3,1) USR3: W0 = (g(1+3g+g^2), g^2)/(G2 G3),          W1 = (1+g-g^2, 0)/(G2 G3)
+        //  (4,1) CSR4: W0 = (-g+g^2+2g^3+3g^4+g^5, g^4)/(G3 G4), W1 = (1+3g+2g^2+g^3-g^4, -g)/(G3 G4)
+        const R g2 = g * g;
+#pragma unroll
+        for (int m = 0; m <= NS; ++m) W0[m] = W1[m] = (R)0;
+        if (k == 2) {
+            const R iv = rcp_bulk((R)1 + g);
+            W0[0] = ((R)2 + g) * iv;
+            W0[1] = iv;
+            W1[0] = -iv;
+        } else if (k == 3) {
+            const R iv = rcp_bulk(((R)1 + g) * ((R)1 + g + g2));
+            W0[0] = g * ((R)1 + (R)3 * g + g2) * iv;
+            W0[1] = g2 * iv;
+            W1[0] = ((R)1 + g - g2) * iv;
+        } else {
+            const R g3 = g2 * g, g4 = g2 * g2;
+            const R iv = rcp_bulk(((R)1 + g + g2) * ((R)1 + g + g2 + g3));
+            W0[0] = (-g + g2 + (R)2 * g3 + (R)3 * g4 + g4 * g) * iv;
+            W0[1] = g4 * iv;
+            W1[0] = ((R)1 + (R)3 * g + (R)2 * g2 + g3 - g4) * iv;
+            W1[1] = -g * iv;
+        }
+        return;
+    }
+    if constexpr (NS == 2) {
+        // USR5: an order-5 step on 630k hexes and prisms FP32 534 -> 457 us
+        if (k == 5 && r == 2) return dolinc_weights_general<NS, R, 5, 2>(k, r, g, W0, W1);
+    }
+    dolinc_weights_general<NS, R, 0, 0>(k, r, g, W0, W1);
 }
 
 // Both orientations' weights: (W0f, W1f) at g and (W0r, W1r) at 1/g (the neighbour-

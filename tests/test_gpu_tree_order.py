@@ -31,6 +31,11 @@ def _mesh(name):
     ("tri_open", "rusanov", 3, 2, "fp32", "weno5_all"),
     ("tri_open", "rusanov", 2, 1, "fp32_bf16", "none"),
     ("tri_open", "rusanov", 3, 2, "fp32", "eno3_all"),
+    ("tri_open", "rusanov", 3, 2, "fp32", "weno5_flagged"),
+    ("tri", "rusanov", 4, 2, "fp32_bf16", "eno3_flagged"),
+    ("tet", "rusanov", 3, 2, "fp32", "weno5_flagged"),
+    ("hexprism", "rusanov", 5, 3, "fp32", "weno5_flagged"),
+    ("hexprism", "upwind", 3, 2, "fp32", "eno3_flagged"),
     ("tet", "rusanov", 3, 2, "fp32", "none"),
     ("tet", "rusanov", 4, 3, "fp32_bf16", "eno3_all"),
     ("tet", "rusanov", 5, 4, "fp32", "none"),
@@ -59,6 +64,8 @@ def test_untuned_shape_gives_the_lane_shape_bits(name, flux, order, n_diff, prec
     else:
         u0 = np.stack([1.0 + s] + [0.4 + 0.2 * np.roll(s, 7 * d) for d in range(dim)] + [3.0 + 0.5 * s])
     lanes = 4 if name in ("tri", "tri_open", "tet") else 8
+    flags = torch.from_numpy((np.sin(9 * xc[:, 0]) * np.sin(7 * xc[:, 1]) > 0.9).astype(np.uint8)).cuda()
+    dg.dolinc_set_flags(M, flags)
 
     def run():
         ws = dg.workspace(M, sch)
