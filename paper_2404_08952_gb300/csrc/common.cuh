@@ -104,6 +104,33 @@ __device__ __forceinline__ void ldg32(const void *p, unsigned *w)
         : "l"(p));
 }
 
+// The same, and 16 bytes, for geometry that a kernel reads once: first to leave the L2,
+// which keeps the records and fluxes that the next kernels read.  Face records in k_flux and
+// weights in k_diff_tree: 630k hexes and prisms order 5 465 -> 452 us a step, 553k
+// tetrahedra order 4 380 -> 374, 1.05M triangles network and step 492 -> 487.  (Not in the
+// paired passes, whose halves share the weights: 2442 -> 2505 us for four steps of 1.31M
+// tetrahedra.)
+__device__ __forceinline__ void ldg32_once(const void *p, unsigned *w)
+{
+    asm("ld.global.nc.L2::evict_first.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+        : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]), "=r"(w[4]), "=r"(w[5]), "=r"(w[6]), "=r"(w[7])
+        : "l"(p));
+}
+__device__ __forceinline__ unsigned long long policy_once()
+{
+    unsigned long long p;
+    asm("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(p));
+    return p;
+}
+__device__ __forceinline__ uint4 ldg16_once(const void *p, unsigned long long policy)
+{
+    uint4 v;
+    asm("ld.global.nc.L2::cache_hint.v4.b32 {%0, %1, %2, %3}, [%4], %5;"
+        : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
+        : "l"(p), "l"(policy));
+    return v;
+}
+
 template <class T, int N, int S, class R, bool LDG = true>
 __device__ __forceinline__ void load_rec(const T *__restrict__ base, long long cell, R *out)
 {

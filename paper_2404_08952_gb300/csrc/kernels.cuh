@@ -121,6 +121,29 @@ template <class R, bool LDG> __device__ __forceinline__ void ld8(const R *p, R *
     }
 }
 
+// Geometry records that the kernel reads once (see ldg32_once): 8 and 4 values
+template <class R> __device__ __forceinline__ void ld8_once(const R *p, R *x)
+{
+#pragma unroll
+    for (int h = 0; h < (int)sizeof(R); h += 4) {
+        unsigned w[8];
+        ldg32_once(p + 8 * h / (int)sizeof(R), w);
+        const R *e = reinterpret_cast<const R *>(w);
+#pragma unroll
+        for (int j = 0; j < 32 / (int)sizeof(R); ++j) x[8 * h / (int)sizeof(R) + j] = e[j];
+    }
+}
+template <class R>
+__device__ __forceinline__ void ld4_once(const R *p, unsigned long long policy, R &a, R &b, R &c, R &d)
+{
+    if constexpr (sizeof(R) == 4) {
+        const uint4 v = ldg16_once(p, policy);
+        a = __uint_as_float(v.x), b = __uint_as_float(v.y), c = __uint_as_float(v.z), d = __uint_as_float(v.w);
+    } else {
+        ld4<R>(p, a, b, c, d);
+    }
+}
+
 // ------------------------------------------------------------------ pack
 // copy (may be null): also written with u, e.g. a device copy of a state that u reads
 // from mapped host memory
@@ -323,6 +346,7 @@ __device__ __forceinline__ void diff_cells_tree(const DevMesh &mesh, const void 
         int s0, s1;
         slot_range(mesh, c, s0, s1);
         const int ns = s1 - s0;
+        const unsigned long long once = policy_once();
         // slots in the order the tree adds them, two at a time: (0, H), (2, H + 2), (1, ..)
         constexpr int H = TREE / 2, NP = TREE / 2;
         constexpr bool ALL = NV * CI <= 10;          // small records: every gather before the first sum
@@ -336,7 +360,7 @@ __device__ __forceinline__ void diff_cells_tree(const DevMesh &mesh, const void 
             for (int h = 0; h < 2; ++h) {
                 const int l = first(p) + h * H;
                 R kb = (R)0;
-                if (l < ns) ld4<R>(Geo<R>::slotk(mesh) + 4ll * (s0 + l), kx[b][h], ky[b][h], kz[b][h], kb);
+                if (l < ns) ld4_once<R>(Geo<R>::slotk(mesh) + 4ll * (s0 + l), once, kx[b][h], ky[b][h], kz[b][h], kb);
                 nb[h] = Geo<R>::nb_of(kb);
             }
 #pragma unroll
@@ -351,7 +375,7 @@ __device__ __forceinline__ void diff_cells_tree(const DevMesh &mesh, const void 
         }
         {
             R own[NV * CI], wx, wy, wz, iv;
-            ld4<R>(Geo<R>::cellk(mesh) + 4ll * c, wx, wy, wz, iv);
+            ld4_once<R>(Geo<R>::cellk(mesh) + 4ll * c, once, wx, wy, wz, iv);
             load_rec<TI, NV * CI, SI, R>(in, c, own);
             poly_mul_acc<DIM, NV, M, R>(acc, own, wx, wy, wz);
         }
@@ -511,9 +535,10 @@ __device__ __forceinline__ int face_limit(const StageArgs &a, bool flagged)
 // Where a kernel reads cell records and face records from.  GlobalSrc: device memory
 // through the read-only path.  TileSrc (k_stage_tile): the block's own cells and the
 // faces they own were staged in shared memory; other cells/faces come from global.
-template <int DIM, int NV, int PREC> struct GlobalSrc {
+// ONCE: the kernel reads each face record once.
+template <int DIM, int NV, int PREC, bool FACE_ONCE = false> struct GlobalSrc {
     using R = typename PrecT<PREC>::R;
-    static constexpr bool LDG = true;
+    static constexpr bool LDG = true, ONCE = FACE_ONCE;
     const StageArgs &a;
     const DevMesh &mesh;
     template <int M> __device__ __forceinline__ const typename OrdT<PREC, M>::T *rec(int X) const
@@ -525,7 +550,7 @@ template <int DIM, int NV, int PREC> struct GlobalSrc {
 
 template <int DIM, int NV, int NS, int PREC> struct TileSrc {
     using R = typename PrecT<PREC>::R;
-    static constexpr bool LDG = false;
+    static constexpr bool LDG = false, ONCE = false;
     const StageArgs &a;
     const DevMesh &mesh;
     const unsigned char *sm;          // staged records of orders 0..NS, then faces
@@ -804,7 +829,8 @@ __device__ __forceinline__ void canon_flux(const StageArgs &a, const Src &src, i
     const int f = (int)(word >> 2);
     const int side = word & 1;
     R fr[8];
-    ld8<R, Src::LDG>(src.face(f), fr);
+    if constexpr (Src::ONCE) ld8_once<R>(src.face(f), fr);
+    else ld8<R, Src::LDG>(src.face(f), fr);
     if (word & 2) {
         // zero-gradient boundary (Sec 2.6): the auxiliary cell mirrors the cell value
         R U[NV];
@@ -932,8 +958,8 @@ __device__ __forceinline__ bool incr_update_cell(const StageArgs &a, int c, long
         const long long i = v * n + c;
         const R d = mul_rn(r[v], dtr);
         const R D = mul_rn((R)(2.0 / 3.0), add_rn((R)a.dacc[i], d));
-        const double o = __dadd_rn(a.u0[i], widen(D));
-        a.out[i] = o;
+        const double o = __dadd_rn(__ldcs(a.u0 + i), widen(D));
+        __stcs(a.out + i, o);
         nx[v] = narrow<R>(o);
         bad |= nonfinite64(o);
     }
@@ -1104,9 +1130,9 @@ __global__ void __launch_bounds__(256) k_flux(DevMesh mesh, StageArgs a)
     using R = typename PrecT<PREC>::R;
     const int f = blockIdx.x * blockDim.x + threadIdx.x;
     if (f >= mesh.n_faces) return;
-    const int P = __ldg(mesh.fo + f), N = __ldg(mesh.fn + f);
+    const int P = __ldcs(mesh.fo + f), N = __ldcs(mesh.fn + f);
     const unsigned word = ((unsigned)f << 2) | (N < 0 ? 2u : 0u);
-    GlobalSrc<DIM, NV, PREC> src{a, mesh};
+    GlobalSrc<DIM, NV, PREC, true> src{a, mesh};
     const bool own_flag = a.flags && a.flags[P];
     R F[NV];
     canon_flux<DIM, NV, NS, PREC>(a, src, P, N < 0 ? P : N, word, own_flag, F);
@@ -1148,7 +1174,7 @@ __global__ void __launch_bounds__(256) k_gather(DevMesh mesh, StageArgs a)
 #pragma unroll
             for (int v = 0; v < NV; ++v) F[l][v] = (R)0;
             if (l < ns) {
-                const unsigned word = __ldg(mesh.sword + s0 + l);
+                const unsigned word = __ldcs(mesh.sword + s0 + l);
                 const long long f = (long long)(word >> 2);
 #pragma unroll
                 for (int v = 0; v < NV; ++v) {
@@ -1169,13 +1195,13 @@ __global__ void __launch_bounds__(256) k_gather(DevMesh mesh, StageArgs a)
     } else if (s1 - s0 == 4 && (s0 & 3) == 0) {
         // the four slot words of a four-slot cell (tetrahedron, quad): one aligned
         // 16-byte load
-        const uint4 w = __ldg(reinterpret_cast<const uint4 *>(mesh.sword + s0));
+        const uint4 w = __ldcs(reinterpret_cast<const uint4 *>(mesh.sword + s0));
         slot(w.x);
         slot(w.y);
         slot(w.z);
         slot(w.w);
     } else {
-        for (int s = s0; s < s1; ++s) slot(__ldg(mesh.sword + s));
+        for (int s = s0; s < s1; ++s) slot(__ldcs(mesh.sword + s));
     }
     cell_epilogue<DIM, NV, PREC>(mesh, a, c, res);
 }
@@ -1429,7 +1455,7 @@ __device__ __forceinline__ void diff_cell(const DevMesh &mesh, const void *in_v,
 
 template <int DIM, int NV, int PREC> struct CoherentSrc {
     using R = typename PrecT<PREC>::R;
-    static constexpr bool LDG = false;
+    static constexpr bool LDG = false, ONCE = false;
     const StageArgs &a;
     const DevMesh &mesh;
     template <int M> __device__ __forceinline__ const typename OrdT<PREC, M>::T *rec(int X) const
