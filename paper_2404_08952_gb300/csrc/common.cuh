@@ -526,6 +526,36 @@ __device__ __forceinline__ void dolinc_weights_both(int k, int r, R g, R *W0f, R
     dolinc_weights<NS, R>(k, r, rcp_bulk(g), W0r, W1r);
 }
 
+// The closed first-order stencils (k = 2, 3, 4; r = 1) in one orientation: left (upwind cell
+// the owner, weights at g) or not (at 1/g, over the same denominator, see
+// dolinc_weights_both).  Face value = iv (A up0 + C down0 + B up1 + D down1), the first-order
+// terms negated by the caller where the upwind cell is the neighbour.
+template <class R>
+__device__ __forceinline__ void upwind_weights(int k, R g, bool left, R &A, R &B, R &C, R &D, R &iv)
+{
+    const R one = (R)1, g2 = g * g;
+    D = (R)0;
+    if (k == 2) {
+        iv = rcp_bulk(one + g);
+        A = left ? (R)2 + g : fma((R)2, g, one);
+        B = left ? one : g;
+        C = -B;
+    } else if (k == 3) {
+        iv = rcp_bulk((one + g) * (one + g + g2));
+        const R q = fma((R)3, g, one + g2);
+        A = left ? g * q : q;
+        B = left ? g2 : g;
+        C = left ? one + g - g2 : g * (g2 + g - one);
+    } else {
+        const R g3 = g2 * g, g4 = g2 * g2;
+        iv = rcp_bulk((one + g + g2) * (one + g + g2 + g3));
+        A = left ? g * fma(g3, g, fma((R)3, g3, fma((R)2, g2, g - one))) : fma((R)3, g, one) + fma((R)2, g2, g3 - g4);
+        B = left ? g4 : g;
+        C = left ? fma((R)3, g, one) + fma((R)2, g2, g3 - g4) : g * fma(g3, g, fma((R)3, g3, fma((R)2, g2, g - one)));
+        D = left ? -g : -g4;
+    }
+}
+
 // ------------------------------------------------------------------ lane groups
 // Sum of v[0..P) over the LPC lanes of an aligned group (LPC a power of two dividing
 // 32), by recursive halving: on return lane j of the group holds the total of

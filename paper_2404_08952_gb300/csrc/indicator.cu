@@ -277,8 +277,9 @@ __device__ __forceinline__ void mma_bf16(float *d, const uint32_t *a, uint2 b)
 // The tile's inputs are staged as bf16 pairs, 12 words per cell (rows of 12 words put the
 // 32 words of an A fragment in distinct banks).  FUSED: they are not read from x but
 // gathered (gather24_cell, one cell per lane).
-// Bound: the tensor pipe and the shared-memory reads.  1.05M triangles, fused: see the
-// table in the design notes for the time; 16 cells per tile took 121 us.
+// Bound: latency of the gathers and of dependent MMAs (tensor pipe 42% busy, 16 warps per
+// SM).  1.05M triangles, fused: 121 us with 16 cells per tile, 95 with 32 at 160 registers,
+// 76 at 128 (four blocks per SM).
 constexpr int XW = MLP_IN / 2;
 
 template <bool FUSED>

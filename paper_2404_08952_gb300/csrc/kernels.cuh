@@ -572,7 +572,8 @@ template <int DIM, int NV, int NS, int PREC> struct TileSrc {
 };
 
 // phi^(m) of every variable of cell X along the monomials of d (m = 0..NS)
-template <int DIM, int NV, int NS, int PREC, int M, class Src>
+// PRE: the monomials already carry the factor 2^m.
+template <int DIM, int NV, int NS, int PREC, int M, bool PRE = false, class Src>
 __device__ __forceinline__ void contract_order(const Src &src, int X, const typename PrecT<PREC>::R *mono,
                                                typename PrecT<PREC>::R (*ph)[NS + 1])
 {
@@ -587,11 +588,11 @@ __device__ __forceinline__ void contract_order(const Src &src, int X, const type
         R s = (R)0;
 #pragma unroll
         for (int q = 0; q < C; ++q) s = fma(rec[v * C + q], mono[mo + q], s);
-        ph[v][M] = s * (R)(1 << M);
+        ph[v][M] = PRE ? s : s * (R)(1 << M);
     }
 }
 
-template <int DIM, int NV, int NS, int PREC, class Src>
+template <int DIM, int NV, int NS, int PREC, bool PRE = false, class Src>
 __device__ __forceinline__ void contract_cell(const Src &src, int X, const typename PrecT<PREC>::R *mono,
                                               typename PrecT<PREC>::R (*ph)[NS + 1])
 {
@@ -603,7 +604,7 @@ __device__ __forceinline__ void contract_cell(const Src &src, int X, const typen
 #pragma unroll
         for (int v = 0; v < NV; ++v) ph[v][0] = rec[v];
     }
-    if constexpr (NS >= 1) contract_order<DIM, NV, NS, PREC, 1>(src, X, mono, ph);
+    if constexpr (NS >= 1) contract_order<DIM, NV, NS, PREC, 1, PRE>(src, X, mono, ph);
     if constexpr (NS >= 2) contract_order<DIM, NV, NS, PREC, 2>(src, X, mono, ph);
     if constexpr (NS >= 3) contract_order<DIM, NV, NS, PREC, 3>(src, X, mono, ph);
     if constexpr (NS >= 4) contract_order<DIM, NV, NS, PREC, 4>(src, X, mono, ph);
@@ -706,9 +707,51 @@ __device__ __forceinline__ void face_states_dolinc(const StageArgs &a, const Src
     R mono[NM];
     monomials<DIM, NS, R>(fr[0], fr[1], fr[2], mono);
     R phP[NV][NS + 1], phN[NV][NS + 1];
+    const R g = fr[3];
+    // FP64 with the closed first-order stencils: two FP64 operations per clock and SM bound
+    // the kernel, so the factor 2 of the first order goes into its monomials, terms with a
+    // zero weight are left out, and the one orientation an upwind face needs is chosen by
+    // selects on polynomials that share a reciprocal (each branch of a warp cost its own
+    // weights).  The same values up to the rounding of the last place.  A residual on 340k
+    // hexes and prisms 183 -> 157 us, an Euler step on 271k tetrahedra 1193 -> 1133 us.
+    if constexpr (NS == 1 && sizeof(R) == 8) {
+        if (a.r == 1 && a.k >= 2 && a.k <= 4) {
+#pragma unroll
+            for (int q = 1; q < NM; ++q) mono[q] *= (R)2;
+            contract_cell<DIM, NV, NS, PREC, true>(src, P, mono, phP);
+            contract_cell<DIM, NV, NS, PREC, true>(src, N, mono, phN);
+            const bool k4 = a.k == 4;
+            if constexpr (UPWIND_ONLY) {
+                R A, B, C, D, iv;
+                upwind_weights<R>(a.k, g, want_left, A, B, C, D, iv);
+#pragma unroll
+                for (int v = 0; v < NV; ++v) {
+                    const R u0 = want_left ? phP[v][0] : phN[v][0], d0 = want_left ? phN[v][0] : phP[v][0];
+                    const R u1 = want_left ? phP[v][1] : -phN[v][1], d1 = want_left ? phN[v][1] : -phP[v][1];
+                    R s = fma(B, u1, fma(C, d0, A * u0));
+                    if (k4) s = fma(D, d1, s);
+                    UL[v] = UR[v] = s * iv;
+                }
+            } else {
+                R W0[2], W1[2], V0[2], V1[2];
+                dolinc_weights_both<1, R>(a.k, a.r, g, W0, W1, V0, V1);
+#pragma unroll
+                for (int v = 0; v < NV; ++v) {
+                    R l = fma(W0[1], phP[v][1], fma(W0[0], phP[v][0], W1[0] * phN[v][0]));
+                    R q = fma(-V0[1], phN[v][1], fma(V0[0], phN[v][0], V1[0] * phP[v][0]));
+                    if (k4) {
+                        l = fma(W1[1], phN[v][1], l);
+                        q = fma(-V1[1], phP[v][1], q);
+                    }
+                    UL[v] = l;
+                    UR[v] = q;
+                }
+            }
+            return;
+        }
+    }
     contract_cell<DIM, NV, NS, PREC>(src, P, mono, phP);
     contract_cell<DIM, NV, NS, PREC>(src, N, mono, phN);
-    const R g = fr[3];
     if constexpr (NS >= 2) {
         if (lim == LIM_ENO3) {
 #pragma unroll
