@@ -211,7 +211,10 @@ dolinc_status dolinc_rk_stage(dolinc_mesh *mesh, const dolinc_scheme *scheme, do
  * equivalent increment form: with d_k = dt R(u_k), u1 = u0 + D0, u2 = u0 + D1 and
  * u^{n+1} = u0 + (2/3)(D1 + d2), where D0 = d0, D1 = (D0 + d1)/4 are kept per cell in
  * the bulk precision; the stage inputs exist only as bulk-precision records and the
- * FP64 state receives one add per step. */
+ * FP64 state receives one add per step.
+ * Untuned steps of a small mesh (up to 40000 cells, stencil order 1, n_diff <= 2) run in
+ * one cooperative launch whose grid barriers wait a bounded time: a wait that gives up is
+ * reported as DOLINC_ERR_DEVICE_TIMEOUT by dolinc_sync_status and leaves u_dev undefined. */
 dolinc_status dolinc_rk_step(dolinc_mesh *mesh, const dolinc_scheme *scheme, double dt, double *u_dev,
                              void *ws_dev, size_t ws_bytes, dolinc_stream stream);
 
