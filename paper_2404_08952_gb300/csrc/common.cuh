@@ -116,11 +116,13 @@ __device__ __forceinline__ void ldg32_once(const void *p, unsigned *w)
         : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]), "=r"(w[4]), "=r"(w[5]), "=r"(w[6]), "=r"(w[7])
         : "l"(p));
 }
-__device__ __forceinline__ unsigned long long policy_once()
+// (first: false where the whole stage fits the L2 and the next stage finds the weights there)
+__device__ __forceinline__ unsigned long long policy_once(bool first)
 {
-    unsigned long long p;
+    unsigned long long p, q;
     asm("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(p));
-    return p;
+    asm("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(q));
+    return first ? p : q;
 }
 __device__ __forceinline__ uint4 ldg16_once(const void *p, unsigned long long policy)
 {

@@ -346,7 +346,9 @@ __device__ __forceinline__ void diff_cells_tree(const DevMesh &mesh, const void 
         int s0, s1;
         slot_range(mesh, c, s0, s1);
         const int ns = s1 - s0;
-        const unsigned long long once = policy_once();
+        // 2^20 slots: a stage of such a mesh moves about 100 MB (181k triangles, 0.5M slots,
+        // criterion and WENO5 step 194 us; evict-first 205)
+        const unsigned long long once = policy_once(mesh.n_slots >= (1 << 20));
         // slots in the order the tree adds them, two at a time: (0, H), (2, H + 2), (1, ..)
         constexpr int H = TREE / 2, NP = TREE / 2;
         constexpr bool ALL = NV * CI <= 10;          // small records: every gather before the first sum
