@@ -410,6 +410,11 @@ dolinc_status dolinc_set_flags(dolinc_mesh *mesh, const uint8_t *flags_dev);
  * values.  Batches take no such meshes. */
 dolinc_status dolinc_set_boundary_values(dolinc_mesh *mesh, int nv, const double *values_host);
 
+/* Polls that a grid-barrier wait of the one-launch steps of small meshes (dolinc_rk_step)
+ * makes before it gives up (default 2^22).  0 makes a wait give up at its first poll: a
+ * way to exercise the timeout path. */
+dolinc_status dolinc_mesh_set_spin_limit(dolinc_mesh *mesh, unsigned polls);
+
 /* Synchronises `stream`, reads and clears the device status word in ws_dev:
  * DOLINC_ERR_NONFINITE if a stage wrote NaN/Inf since the last call,
  * DOLINC_ERR_DEVICE_TIMEOUT if a bounded wait gave up, else DOLINC_OK. */

@@ -37,7 +37,7 @@ ABI_SYMBOLS = (
     "dolinc_mesh_set_skew_correction", "dolinc_implicit_create", "dolinc_implicit_destroy",
     "dolinc_implicit_set_solver", "dolinc_implicit_step", "dolinc_implicit_info", "dolinc_implicit_rows",
     "dolinc_implicit_set_layout", "dolinc_implicit_layout",
-    "dolinc_last_error",
+    "dolinc_mesh_set_spin_limit", "dolinc_last_error",
 )
 KERNEL_KINDS = ("pack", "diff1", "diff2", "diff3", "diff4", "stage", "faces", "diff_pair", "solve")
 
@@ -111,7 +111,7 @@ def load(path=LIB_PATH):
             "dolinc_mesh_create_part": [P, P, I, I, P], "dolinc_mesh_part_sizes": [P, P],
             "dolinc_part_step_begin": [P, P, D, P, P, S, P, P],
             "dolinc_part_step_continue": [P, P, P, S, P, P],
-            "dolinc_mesh_set_skew_correction": [P, I],
+            "dolinc_mesh_set_skew_correction": [P, I], "dolinc_mesh_set_spin_limit": [P, C.c_uint],
             "dolinc_implicit_create": [P, P, D, D, P], "dolinc_implicit_destroy": [P],
             "dolinc_implicit_set_solver": [P, D, I, C.c_uint, I], "dolinc_implicit_step": [P, P, I, P, S, P],
             "dolinc_implicit_info": [P, P], "dolinc_implicit_rows": [P, P, P, P, P],
@@ -296,6 +296,11 @@ class Mesh:
         d = np.zeros((self.n_faces, 3))
         _check(load().dolinc_mesh_geometry(self.handle, _ptr(V), _ptr(xc), _ptr(S), _ptr(w), _ptr(d)))
         return dict(V=V, xc=xc, S=S, w=w, d=d)
+
+
+def dolinc_mesh_set_spin_limit(mesh, polls=1 << 22):
+    """Polls a grid-barrier wait of the one-launch steps of small meshes makes."""
+    _check(load().dolinc_mesh_set_spin_limit(mesh.handle, int(polls)))
 
 
 def dolinc_mesh_set_skew_correction(mesh, enable=True):

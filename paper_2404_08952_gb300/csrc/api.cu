@@ -100,7 +100,8 @@ struct dolinc_mesh {
     int bv_nv = 0;                     // variables of the boundary values set (0: none yet)
     std::vector<int32_t> bidx_h;       // host copy of DevMesh::bidx
     int max_faces = 0;                 // largest number of slots of a cell
-    unsigned *steps_bar = nullptr;     // grid-barrier words of k_steps_small, zero between launches
+    unsigned *steps_bar = nullptr;     // BAR_WORDS grid-barrier words of k_steps_small, zero between launches
+    unsigned steps_spin = 1u << 22;    // polls one of its barrier waits makes before giving up
     std::map<std::string, Tune> tuned;  // launch shapes chosen by dolinc_autotune, per scheme
     // per-kernel timing (dolinc_profile_enable)
     bool prof = false;
@@ -620,7 +621,7 @@ dolinc_status upload_mesh(dolinc_mesh *m)
         (st = upload(m, ff, &d.face_flip)) || (st = upload(m, fown, &d.fown)))
         return st;
     const unsigned *bar = nullptr;
-    if ((st = upload(m, std::vector<unsigned>(64, 0u), &bar))) return st;
+    if ((st = upload(m, std::vector<unsigned>(BAR_WORDS, 0u), &bar))) return st;
     m->steps_bar = const_cast<unsigned *>(bar);
     return DOLINC_OK;
 }
@@ -833,7 +834,7 @@ cudaError_t small_steps(dolinc_mesh *m, const PathFns *p, const dolinc_scheme *s
     q.n_diff = s->n_diff;
     q.n_steps = n_steps;
     q.bar = m->steps_bar;
-    q.spin_limit = 1u << 22;
+    q.spin_limit = m->steps_spin;
     return p->steps_small(m->d, q, m->max_faces <= 4 ? 4 : 8, cs);
 }
 
@@ -1460,6 +1461,7 @@ dolinc_status batch_launch_step(dolinc_batch *bt, const dolinc_scheme *s, const 
         b.n_diff = s->n_diff;
         b.cell_mesh = bt->cell_mesh;
         b.dt_tab = dt;
+        static_assert(256 + 4 * BAR_WORDS <= 1024, "barrier words within the cleared head of the workspace");
         b.bar = reinterpret_cast<unsigned *>(B(ws, L.status + 256));
         b.spin_limit = bt->spin_limit;
         cudaError_t e = bf->launch(m->d, a, b, bt->grid, bt->block, cs);
@@ -1661,6 +1663,13 @@ dolinc_status dolinc_set_flags(dolinc_mesh *m, const uint8_t *flags)
 {
     if (!m) return fail(DOLINC_ERR_INVALID_ARG, "null mesh");
     m->flags = flags;
+    return DOLINC_OK;
+}
+
+dolinc_status dolinc_mesh_set_spin_limit(dolinc_mesh *m, unsigned polls)
+{
+    if (!m) return fail(DOLINC_ERR_INVALID_ARG, "null mesh");
+    m->steps_spin = polls;
     return DOLINC_OK;
 }
 

@@ -558,6 +558,10 @@ __device__ __forceinline__ void upwind_weights(int k, R g, bool left, R &A, R &B
     }
 }
 
+// ------------------------------------------------------------------ grid barriers
+// Words of a grid barrier of a cooperative launch, on separate 128-byte lines.
+enum { BAR_ARRIVED = 0, BAR_LEFT = 32, BAR_ABORT = 64, BAR_WORDS = 96 };
+
 // ------------------------------------------------------------------ lane groups
 // Sum of v[0..P) over the LPC lanes of an aligned group (LPC a power of two dividing
 // 32), by recursive halving: on return lane j of the group holds the total of

@@ -1416,26 +1416,25 @@ struct BatchArgs {
 };
 
 // Grid barrier of a cooperative launch: arrive, then wait until every block has arrived
-// `round` times (rounds count from 1 in each launch).  bar[0] arrivals, bar[32] blocks that
-// left, bar[64] abort.  False if the wait gave up here or elsewhere.
+// `round` times (rounds count from 1 in each launch).  bar: BAR_WORDS words.  False if the
+// wait gave up here or elsewhere; either sets status bit 1, so that no launch ends early
+// without a report.
 __device__ __forceinline__ bool grid_sync(unsigned *bar, unsigned round, unsigned *status, unsigned limit)
 {
     __shared__ int ok;
     __syncthreads();
     if (threadIdx.x == 0) {
         const unsigned target = round * gridDim.x;
-        volatile unsigned *abort = bar + 64;
-        asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(bar) : "memory");
+        volatile unsigned *abort = bar + BAR_ABORT;
+        asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(bar + BAR_ARRIVED) : "memory");
         unsigned it = 0, v;
         ok = 1;
         for (;;) {
-            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(bar) : "memory");
+            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(bar + BAR_ARRIVED) : "memory");
             if ((int)(v - target) >= 0) break;
-            if (++it > limit) {
-                atomicOr(status, 2u);
-                *abort = 1u;
-            }
+            if (++it > limit) *abort = 1u;
             if (it > limit || ((it & 63u) == 0 && *abort)) {
+                atomicOr(status, 2u);
                 ok = 0;
                 break;
             }
@@ -1451,10 +1450,10 @@ __device__ __forceinline__ void grid_leave(unsigned *bar, bool clear_abort)
     __syncthreads();
     if (threadIdx.x == 0) {
         __threadfence();
-        if (atomicAdd(bar + 32, 1u) == gridDim.x - 1) {
-            bar[0] = 0;
-            bar[32] = 0;
-            if (clear_abort) bar[64] = 0;
+        if (atomicAdd(bar + BAR_LEFT, 1u) == gridDim.x - 1) {
+            bar[BAR_ARRIVED] = 0;
+            bar[BAR_LEFT] = 0;
+            if (clear_abort) bar[BAR_ABORT] = 0;
         }
     }
 }
@@ -1520,7 +1519,7 @@ __global__ void __launch_bounds__(256, (NV == 1 && NS == 1 && PREC != PREC_F64) 
     const int n = mesh.n_cells;
     constexpr int S0 = ord_stride<DIM, NV, 0, PREC>();
     unsigned round = 0;
-    bool ok = !*(volatile unsigned *)(b.bar + 64);
+    bool ok = !*(volatile unsigned *)(b.bar + BAR_ABORT);
     auto sync = [&] { ok = ok && grid_sync(b.bar, ++round, a.status, b.spin_limit); };
     if (ok && b.pack_src) {
         for (int c = tid; c < n; c += nthr) {
@@ -1541,7 +1540,7 @@ __global__ void __launch_bounds__(256, (NV == 1 && NS == 1 && PREC != PREC_F64) 
             for (int c = tid; c < n; c += nthr) diff_cell<DIM, NV, 2, PREC>(mesh, b.ord[1], b.ord[2], c);
             sync();
         }
-    if (!ok || *(volatile unsigned *)(b.bar + 64)) {     // a barrier gave up: leave the state untouched
+    if (!ok || *(volatile unsigned *)(b.bar + BAR_ABORT)) {     // a barrier gave up: leave the state untouched
         grid_leave(b.bar, false);
         return;
     }
@@ -1582,7 +1581,7 @@ __global__ void __launch_bounds__(256, (NV == 1 && NS == 1 && PREC != PREC_F64) 
             for (int v = 0; v < NV; ++v) flux[(long long)v * nf + i] = F[v];
         }
         sync();
-        if (!ok || *(volatile unsigned *)(b.bar + 64)) {     // a barrier gave up: leave the state untouched
+        if (!ok || *(volatile unsigned *)(b.bar + BAR_ABORT)) {     // a barrier gave up: leave the state untouched
             grid_leave(b.bar, false);
             return;
         }
