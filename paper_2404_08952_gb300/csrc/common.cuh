@@ -562,6 +562,14 @@ __device__ __forceinline__ void upwind_weights(int k, R g, bool left, R &A, R &B
 // Words of a grid barrier of a cooperative launch, on separate 128-byte lines.
 enum { BAR_ARRIVED = 0, BAR_LEFT = 32, BAR_ABORT = 64, BAR_WORDS = 96 };
 
+// The abort word, the same answer in every thread of the block (all of them call it).
+// Another block may set the word between two threads' reads, and what depends on it leads
+// to block barriers.
+__device__ __forceinline__ bool grid_aborted(const unsigned *bar)
+{
+    return __syncthreads_or(threadIdx.x == 0 && *(volatile const unsigned *)(bar + BAR_ABORT));
+}
+
 // ------------------------------------------------------------------ lane groups
 // Sum of v[0..P) over the LPC lanes of an aligned group (LPC a power of two dividing
 // 32), by recursive halving: on return lane j of the group holds the total of

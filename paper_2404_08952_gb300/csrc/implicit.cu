@@ -557,7 +557,7 @@ template <bool ALL> __global__ void __launch_bounds__(SMB) k_imp_solve_sm(ImpSol
         sc.done = sc.iters = 0;
         sc.status = 0;
     }
-    bool ok = !*(volatile unsigned *)(a.bar + 64);
+    bool ok = !grid_aborted(a.bar);
 
     {
         double red[2] = {0.0, 0.0};

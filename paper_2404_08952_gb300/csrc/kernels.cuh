@@ -1519,7 +1519,7 @@ __global__ void __launch_bounds__(256, (NV == 1 && NS == 1 && PREC != PREC_F64) 
     const int n = mesh.n_cells;
     constexpr int S0 = ord_stride<DIM, NV, 0, PREC>();
     unsigned round = 0;
-    bool ok = !*(volatile unsigned *)(b.bar + BAR_ABORT);
+    bool ok = !grid_aborted(b.bar);
     auto sync = [&] { ok = ok && grid_sync(b.bar, ++round, a.status, b.spin_limit); };
     if (ok && b.pack_src) {
         for (int c = tid; c < n; c += nthr) {
@@ -1540,7 +1540,7 @@ __global__ void __launch_bounds__(256, (NV == 1 && NS == 1 && PREC != PREC_F64) 
             for (int c = tid; c < n; c += nthr) diff_cell<DIM, NV, 2, PREC>(mesh, b.ord[1], b.ord[2], c);
             sync();
         }
-    if (!ok || *(volatile unsigned *)(b.bar + BAR_ABORT)) {     // a barrier gave up: leave the state untouched
+    if (!ok || grid_aborted(b.bar)) {     // a barrier gave up: leave the state untouched
         grid_leave(b.bar, false);
         return;
     }
@@ -1581,7 +1581,7 @@ __global__ void __launch_bounds__(256, (NV == 1 && NS == 1 && PREC != PREC_F64) 
             for (int v = 0; v < NV; ++v) flux[(long long)v * nf + i] = F[v];
         }
         sync();
-        if (!ok || *(volatile unsigned *)(b.bar + BAR_ABORT)) {     // a barrier gave up: leave the state untouched
+        if (!ok || grid_aborted(b.bar)) {     // a barrier gave up: leave the state untouched
             grid_leave(b.bar, false);
             return;
         }

@@ -36,6 +36,17 @@ def test_words_of_the_batch_lie_in_the_cleared_head_of_the_workspace():
     assert off + 4 * (max(_words("kernels.cuh")) + 1) <= 1024
 
 
+def test_a_block_takes_one_answer_from_the_abort_word():
+    """What a block does after reading the abort word leads to block barriers, so one thread
+    reads it for the block (grid_aborted, or thread 0 of a barrier); only a poll whose
+    answer goes through shared memory reads it by itself."""
+    for name in ("kernels.cuh", "implicit.cu"):
+        src = _read(name)
+        reads = [src[:m.start()].rsplit("\n", 1)[1] for m in re.finditer(r"\*\(volatile unsigned \*\)\(", src)]
+        assert all(r.strip() == "if ((it & 63u) == 0 &&" for r in reads), (name, reads)
+        assert "grid_aborted(" in src
+
+
 def test_words_of_the_solver_lie_in_its_control_block():
     src = _read("api.cu")
     ctrl = int(re.search(r"kImpCtrl = (\d+)", src).group(1))
