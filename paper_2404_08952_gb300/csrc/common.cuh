@@ -559,7 +559,8 @@ __device__ __forceinline__ void upwind_weights(int k, R g, bool left, R &A, R &B
 }
 
 // ------------------------------------------------------------------ grid barriers
-// Words of a grid barrier of a cooperative launch, on separate 128-byte lines.
+// Words of a grid barrier of a cooperative launch, on separate 128-byte lines (the arrivals
+// a 64-bit count).
 enum { BAR_ARRIVED = 0, BAR_LEFT = 32, BAR_ABORT = 64, BAR_WORDS = 96 };
 
 // The abort word, the same answer in every thread of the block (all of them call it).

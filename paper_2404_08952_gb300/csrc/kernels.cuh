@@ -1416,28 +1416,34 @@ struct BatchArgs {
 };
 
 // Grid barrier of a cooperative launch: arrive, then wait until every block has arrived
-// `round` times (rounds count from 1 in each launch).  bar: BAR_WORDS words.  False if the
-// wait gave up here or elsewhere; either sets status bit 1, so that no launch ends early
-// without a report.
+// `round` times (rounds count from 1 in each launch).  bar: BAR_WORDS words.  False if a
+// wait gave up, here or elsewhere, and then for every block: the arrivals add 2 each, and a
+// wait that gives up raises an incomplete count to the odd number below its target in one
+// atomic operation, which leaves a complete count alone.  An odd count stays odd, so no
+// block passes that round (the arrivals still to come leave it below `next`), while one
+// that looks late still sees that the rounds before were complete.  Whoever does not pass
+// sets status bit 1, so no launch ends early without a report, and the abort word.
 __device__ __forceinline__ bool grid_sync(unsigned *bar, unsigned round, unsigned *status, unsigned limit)
 {
     __shared__ int ok;
     __syncthreads();
     if (threadIdx.x == 0) {
-        const unsigned target = round * gridDim.x;
-        volatile unsigned *abort = bar + BAR_ABORT;
-        asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(bar + BAR_ARRIVED) : "memory");
-        unsigned it = 0, v;
-        ok = 1;
-        for (;;) {
-            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(bar + BAR_ARRIVED) : "memory");
-            if ((int)(v - target) >= 0) break;
-            if (++it > limit) *abort = 1u;
-            if (it > limit || ((it & 63u) == 0 && *abort)) {
-                atomicOr(status, 2u);
-                ok = 0;
+        unsigned long long *count = reinterpret_cast<unsigned long long *>(bar + BAR_ARRIVED);
+        const unsigned long long target = 2ull * round * gridDim.x, next = target + 2ull * gridDim.x - 1;
+        asm volatile("red.release.gpu.global.add.u64 [%0], 2;" ::"l"(count) : "memory");
+        unsigned long long v;
+        for (unsigned it = 0;;) {
+            asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(count) : "memory");
+            if (v >= target || (v & 1)) break;
+            if (++it > limit) {
+                v = atomicMax(count, target - 1);
                 break;
             }
+        }
+        ok = v >= ((v & 1) ? next : target);
+        if (!ok) {
+            atomicOr(status, 2u);
+            *(volatile unsigned *)(bar + BAR_ABORT) = 1u;
         }
     }
     __syncthreads();
@@ -1451,7 +1457,7 @@ __device__ __forceinline__ void grid_leave(unsigned *bar, bool clear_abort)
     if (threadIdx.x == 0) {
         __threadfence();
         if (atomicAdd(bar + BAR_LEFT, 1u) == gridDim.x - 1) {
-            bar[BAR_ARRIVED] = 0;
+            *reinterpret_cast<unsigned long long *>(bar + BAR_ARRIVED) = 0;
             bar[BAR_LEFT] = 0;
             if (clear_abort) bar[BAR_ABORT] = 0;
         }
@@ -1540,7 +1546,25 @@ __global__ void __launch_bounds__(256, (NV == 1 && NS == 1 && PREC != PREC_F64) 
             for (int c = tid; c < n; c += nthr) diff_cell<DIM, NV, 2, PREC>(mesh, b.ord[1], b.ord[2], c);
             sync();
         }
-    if (!ok || grid_aborted(b.bar)) {     // a barrier gave up: leave the state untouched
+    // Two or three orders above the stencil's: before the stage, so that every barrier comes
+    // before the first write of the output (one such order runs beside the stage)
+    if (NS + 2 <= b.n_diff) {
+        if (ok) {
+            for (int c = tid; c < n; c += nthr) diff_cell<DIM, NV, NS + 1, PREC>(mesh, b.ord[NS], b.ord[NS + 1], c);
+            sync();
+        }
+        if (ok)
+            for (int c = tid; c < n; c += nthr) diff_cell<DIM, NV, NS + 2, PREC>(mesh, b.ord[NS + 1], b.ord[NS + 2], c);
+        if constexpr (NS + 3 <= MAXN)
+            if (NS + 3 <= b.n_diff) {
+                sync();
+                if (ok)
+                    for (int c = tid; c < n; c += nthr)
+                        diff_cell<DIM, NV, NS + 3, PREC>(mesh, b.ord[NS + 2], b.ord[NS + 3], c);
+            }
+    }
+    const bool beside = b.n_diff == NS + 1;
+    if (!ok) {                            // a barrier gave up: leave the output untouched
         grid_leave(b.bar, false);
         return;
     }
@@ -1567,7 +1591,7 @@ __global__ void __launch_bounds__(256, (NV == 1 && NS == 1 && PREC != PREC_F64) 
         // stencil's, which the stage does not read (no barrier between), then the sums
         const int nf = mesh.n_faces;
         R *flux = static_cast<R *>(a.face_flux);
-        const int work = nf + (NS + 1 <= b.n_diff ? n : 0);
+        const int work = nf + (beside ? n : 0);
         for (int i = tid; i < work; i += nthr) {
             if (i >= nf) {
                 diff_cell<DIM, NV, NS + 1, PREC>(mesh, b.ord[NS], b.ord[NS + 1], i - nf);
@@ -1581,7 +1605,7 @@ __global__ void __launch_bounds__(256, (NV == 1 && NS == 1 && PREC != PREC_F64) 
             for (int v = 0; v < NV; ++v) flux[(long long)v * nf + i] = F[v];
         }
         sync();
-        if (!ok || grid_aborted(b.bar)) {     // a barrier gave up: leave the state untouched
+        if (!ok) {
             grid_leave(b.bar, false);
             return;
         }
@@ -1604,7 +1628,7 @@ __global__ void __launch_bounds__(256, (NV == 1 && NS == 1 && PREC != PREC_F64) 
     } else {
         // one pass over the cells (face-centric: 190 us a step on 600k triangles against 178)
         for (int c = tid; c < n; c += nthr) {
-            if (NS + 1 <= b.n_diff) diff_cell<DIM, NV, NS + 1, PREC>(mesh, b.ord[NS], b.ord[NS + 1], c);
+            if (beside) diff_cell<DIM, NV, NS + 1, PREC>(mesh, b.ord[NS], b.ord[NS + 1], c);
             R res[NV];
 #pragma unroll
             for (int v = 0; v < NV; ++v) res[v] = (R)0;
@@ -1622,19 +1646,6 @@ __global__ void __launch_bounds__(256, (NV == 1 && NS == 1 && PREC != PREC_F64) 
             finish(c, res, dtr);
         }
     }
-    // still higher orders, a barrier before each
-    if (NS + 2 <= b.n_diff) {
-        sync();
-        if (ok)
-            for (int c = tid; c < n; c += nthr) diff_cell<DIM, NV, NS + 2, PREC>(mesh, b.ord[NS + 1], b.ord[NS + 2], c);
-    }
-    if constexpr (NS + 3 <= MAXN)
-        if (NS + 3 <= b.n_diff) {
-            sync();
-            if (ok)
-                for (int c = tid; c < n; c += nthr)
-                    diff_cell<DIM, NV, NS + 3, PREC>(mesh, b.ord[NS + 2], b.ord[NS + 3], c);
-        }
     grid_leave(b.bar, false);
 }
 

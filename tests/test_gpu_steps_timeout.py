@@ -88,3 +88,31 @@ def test_every_block_of_a_solve_leaves_on_a_timeout():
         S.step(u, ws)
         assert S.info()["converged"]
         np.testing.assert_array_equal(u.cpu().numpy(), ref.cpu().numpy())
+
+
+@pytest.mark.parametrize("precision,k,r,n_diff", [("fp64", 3, 1, 2), ("fp64", 3, 1, 4), ("fp32", 3, 1, 3),
+                                                  ("fp32", 3, 1, 4), ("fp32", 5, 2, 4)])
+def test_a_batch_step_is_whole_or_leaves_the_state(precision, k, r, n_diff):
+    """Whatever poll limit a launch runs into, a reported timeout leaves the state as it was,
+    and a step that reports none is the step of the normal limit."""
+    bt = dg.Batch([dg.Mesh(synth.tri_mesh(120, 110, 0.2, s)) for s in (1, 2, 3)])
+    sch = dg.Scheme(k=k, r=r, n_diff=n_diff, flux="burgers", nv=1, precision=precision)
+    ws = bt.workspace(sch)
+    u0 = torch.from_numpy(1.0 + 0.1 * np.random.default_rng(6).random((1, sum(M.n_cells for M in bt.meshes)))).cuda()
+    dt = torch.full((3,), 1e-4, dtype=torch.float64, device="cuda")
+    want = u0.clone()
+    bt.rk_step(sch, dt, want, ws, use_graph=False)
+    dg.dolinc_sync_status(bt.meshes[0], ws)
+    gave_up = 0
+    for limit in [0] + list(range(1, 120, 2)):
+        bt.set_spin_limit(limit)
+        u = u0.clone()
+        bt.rk_step(sch, dt, u, ws, use_graph=False)
+        try:
+            dg.dolinc_sync_status(bt.meshes[0], ws)
+            assert torch.equal(u, want), limit
+        except dg.DolincError as e:
+            assert e.status == 5
+            gave_up += 1
+            assert torch.equal(u, u0), limit
+    assert gave_up > 0
