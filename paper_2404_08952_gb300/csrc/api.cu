@@ -1240,6 +1240,7 @@ dolinc_status dolinc_mlp_create(dolinc_mlp **out, uint64_t seed)
     cudaError_t e = cudaSuccess;
     for (float **p : {&m->theta, &m->m, &m->v})
         if (e == cudaSuccess) e = al((void **)p, sizeof(float) * MLP_PARAMS);
+    if (e == cudaSuccess) e = mlp_setup();
     if (e == cudaSuccess) e = al((void **)&m->part, sizeof(float) * MLP_PART * MLP_MAX_PARTS);
     if (e == cudaSuccess) e = al((void **)&m->frag, sizeof(uint2) * N_FRAGS * 32);
     if (e == cudaSuccess) e = cudaMemcpy(m->theta, th.data(), sizeof(float) * MLP_PARAMS, cudaMemcpyHostToDevice);
@@ -1290,6 +1291,8 @@ dolinc_status dolinc_mlp_loss_grad(dolinc_mlp *m, const float *x, const uint8_t 
     if (!m || !x || !y || n <= 0) return fail(DOLINC_ERR_INVALID_ARG, "bad argument");
     cudaStream_t cs = reinterpret_cast<cudaStream_t>(stream);
     const int np = launch_mlp_grad(m->theta, x, y, n, pos_weight, m->part, cs);
+    dolinc_status st = launch_check();
+    if (st) return st;
     launch_mlp_reduce(m->part, np, grad, loss, nullptr, nullptr, nullptr, 0.f, 1, cs);
     return launch_check();
 }
@@ -1300,6 +1303,8 @@ dolinc_status dolinc_mlp_train_step(dolinc_mlp *m, const float *x, const uint8_t
     if (!m || !x || !y || n <= 0) return fail(DOLINC_ERR_INVALID_ARG, "bad argument");
     cudaStream_t cs = reinterpret_cast<cudaStream_t>(stream);
     const int np = launch_mlp_grad(m->theta, x, y, n, pos_weight, m->part, cs);
+    dolinc_status st = launch_check();
+    if (st) return st;                            // no gradient: the weights and the step stay
     m->step += 1;
     launch_mlp_reduce(m->part, np, nullptr, loss, m->theta, m->m, m->v, lr, m->step, cs);
     m->frag_ok = false;
@@ -2147,11 +2152,17 @@ dolinc_status dolinc_implicit_create(dolinc_mesh *m, const dolinc_scheme *s, dou
     CU(cudaGetDevice(&cur));
     CU(cudaSetDevice(m->device));
     CU(cudaDeviceGetAttribute(&imp->sms, cudaDevAttrMultiProcessorCount, m->device));
+    cudaError_t e = imp_sm_setup();
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        cudaSetDevice(cur);
+        return fail(DOLINC_ERR_CUDA, std::string("semi-implicit solve: ") + cudaGetErrorString(e));
+    }
     auto al = [](size_t b) { return (b + 255) / 256 * 256; };
     const size_t n8 = al(8 * (size_t)std::max<int64_t>(imp->n, 1));
     const size_t pb = al(8 * IMP_NRED * (size_t)imp->sms * kImpMaxBlocksPerSm);
     const size_t total = 15 * n8 + pb + kImpCtrl + 256;    // 7 vectors, diag, bscale, R, Rn, un, 3 kept solutions
-    cudaError_t e = cudaMalloc(&imp->mem, total);
+    e = cudaMalloc(&imp->mem, total);
     if (e != cudaSuccess) {
         cudaGetLastError();
         cudaSetDevice(cur);

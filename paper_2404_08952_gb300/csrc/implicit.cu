@@ -728,16 +728,17 @@ int imp_ell_width(int max_slots) { return max_slots <= 4 ? 4 : max_slots <= 6 ? 
 // cells of the largest mesh for which four vectors fit the SMs' shared memory
 int64_t imp_sm_cells(int sms) { return (int64_t)sms * (SM_BYTES / 8 / 4 - 32); }
 
+cudaError_t imp_sm_setup()
+{
+    for (auto k : {k_imp_solve_sm<true>, k_imp_solve_sm<false>}) {
+        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, SM_RED + SM_BYTES);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+}
+
 cudaError_t launch_imp_solve_sm(const ImpSolve &a, int sms, cudaStream_t s)
 {
-    static bool attr = false;   // opt in to more than 48 KB once
-    if (!attr) {
-        for (auto k : {k_imp_solve_sm<true>, k_imp_solve_sm<false>}) {
-            cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, SM_RED + SM_BYTES);
-            if (e != cudaSuccess) return e;
-        }
-        attr = true;
-    }
     // chunks of at least 256 cells, whole warps of them
     const int chunk = std::max(256, ((a.n + sms - 1) / sms + 31) / 32 * 32);
     const int n_sm = std::min(7, SM_BYTES / 8 / chunk);

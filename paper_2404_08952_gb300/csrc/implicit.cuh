@@ -55,6 +55,7 @@ int imp_solve_blocks_per_sm(int ell);
 // shared memory (bar: [32] blocks that left, [64] abort; life[2]: the tag its posts go
 // on from; part: 2 sets of IMP_NRED 16-byte words per SM)
 int64_t imp_sm_cells(int sms);
+cudaError_t imp_sm_setup();      // once per device, before its first launch
 cudaError_t launch_imp_solve_sm(const ImpSolve &a, int sms, cudaStream_t s);
 constexpr int IMP_BLOCK = 256;
 constexpr int IMP_NRED = 4;      // values a grid barrier reduces at most (partials per block)

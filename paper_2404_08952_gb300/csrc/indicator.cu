@@ -698,14 +698,13 @@ void launch_mlp_infer_fused(const uint2 *frag, const float *theta, const DevMesh
     if (blocks < 1) blocks = 1;
     k_mlp_infer<true><<<blocks, 128, 0, s>>>(frag, theta, nullptr, n, logits, flags, m, own);
 }
+cudaError_t mlp_setup()
+{
+    return cudaFuncSetAttribute(k_mlp_grad, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(MlpTile));
+}
 int launch_mlp_grad(const float *theta, const float *x, const uint8_t *y, long long n, float pw, float *part,
                     cudaStream_t s)
 {
-    static bool attr = false;   // opt in to more than 48 KB once
-    if (!attr) {
-        cudaFuncSetAttribute(k_mlp_grad, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(MlpTile));
-        attr = true;
-    }
     const long long tiles = (n + GT - 1) / GT;
     const int grid = (int)(tiles < MLP_MAX_PARTS ? tiles : MLP_MAX_PARTS);
     k_mlp_grad<<<grid, 256, sizeof(MlpTile), s>>>(theta, x, y, n, pw, part);

@@ -39,6 +39,8 @@ void launch_mlp_infer_fused(const uint2 *frag, const float *theta, const DevMesh
 // loss; at most MLP_MAX_PARTS) into part; returns their number.  Then their sum, into
 // grad and *loss where not null, and with theta an Adam step on theta, m and v.
 constexpr int MLP_PART = 9988, MLP_MAX_PARTS = 304;      // 304: two CTAs on each of 152 SMs
+// (mlp_setup: once per device, before its first launch_mlp_grad)
+cudaError_t mlp_setup();
 int launch_mlp_grad(const float *theta, const float *x, const uint8_t *y, long long n, float pos_weight, float *part,
                     cudaStream_t s);
 void launch_mlp_reduce(const float *part, int n_part, float *grad, float *loss, float *theta, float *m, float *v,
