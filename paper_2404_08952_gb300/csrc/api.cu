@@ -152,7 +152,8 @@ struct dolinc_batch {
     int n = 0;
     std::vector<int64_t> cell_off;
     const int32_t *cell_mesh = nullptr;
-    int block = 256, grid = 0;         // persistent launch shape (0: from occupancy)
+    int block = 256, grid = 0;         // persistent launch shape (grid 0: as many blocks as fit)
+    std::map<std::pair<const void *, int>, int> fit;   // resident blocks of each kernel and block size
     unsigned spin_limit = 1u << 23;    // polls a grid-barrier wait makes before giving up
     cudaGraphExec_t exec = nullptr;
     cudaStream_t cap = nullptr;        // private stream the graph is captured on
@@ -1444,7 +1445,7 @@ dolinc_status dolinc_batch_workspace_size(const dolinc_batch *b, const dolinc_sc
 
 namespace {
 dolinc_status batch_launch_step(dolinc_batch *bt, const dolinc_scheme *s, const BatchFns *bf, const double *dt,
-                                double *u, void *ws, const WsLayout &L, cudaStream_t cs)
+                                double *u, void *ws, const WsLayout &L, int grid, cudaStream_t cs)
 {
     static const double A[3] = {0.0, 0.75, 1.0 / 3.0}, Bc[3] = {1.0, 0.25, 2.0 / 3.0};
     dolinc_mesh *m = bt->arena;
@@ -1469,7 +1470,7 @@ dolinc_status batch_launch_step(dolinc_batch *bt, const dolinc_scheme *s, const 
         static_assert(256 + 4 * BAR_WORDS <= 1024, "barrier words within the cleared head of the workspace");
         b.bar = reinterpret_cast<unsigned *>(B(ws, L.status + 256));
         b.spin_limit = bt->spin_limit;
-        cudaError_t e = bf->launch(m->d, a, b, bt->grid, bt->block, cs);
+        cudaError_t e = bf->launch(m->d, a, b, grid, bt->block, cs);
         if (e != cudaSuccess) return fail(DOLINC_ERR_CUDA, std::string("cooperative launch: ") + cudaGetErrorString(e));
         cur = 1 - cur;
     }
@@ -1477,7 +1478,7 @@ dolinc_status batch_launch_step(dolinc_batch *bt, const dolinc_scheme *s, const 
 }
 
 dolinc_status batch_prepare(dolinc_batch *bt, const dolinc_scheme *s, const double *dt, double *u, void *ws,
-                            size_t ws_bytes, WsLayout &L, const BatchFns **bf)
+                            size_t ws_bytes, WsLayout &L, const BatchFns **bf, int &grid)
 {
     dolinc_mesh *m = bt->arena;
     dolinc_status st = check_scheme(m, s);
@@ -1490,13 +1491,17 @@ dolinc_status batch_prepare(dolinc_batch *bt, const dolinc_scheme *s, const doub
     std::call_once(g_once, init_paths);
     *bf = &g_batch[batch_index(m->h.dim, s->nv, ns, s->precision)];
     if (!(*bf)->launch) return fail(DOLINC_ERR_UNSUPPORTED, "no batched kernel for this scheme");
-    if (bt->grid <= 0) {
+    // the kernels of a batch's schemes need different registers: each launch takes what fits
+    // of its own kernel, an autotuned shape at most its grid
+    int &fit = bt->fit[{*bf, bt->block}];
+    if (fit <= 0) {
         int sms = 0;
         CU(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, m->device));
         const int per = (*bf)->blocks_per_sm(bt->block);
         if (per <= 0) return fail(DOLINC_ERR_UNSUPPORTED, "batched kernel does not fit on an SM");
-        bt->grid = per * sms;
+        fit = per * sms;
     }
+    grid = bt->grid > 0 ? std::min(bt->grid, fit) : fit;
     return DOLINC_OK;
 }
 }  // namespace
@@ -1507,14 +1512,15 @@ dolinc_status dolinc_batch_rk_step(dolinc_batch *bt, const dolinc_scheme *s, con
     if (!bt) return fail(DOLINC_ERR_INVALID_ARG, "null batch");
     WsLayout L;
     const BatchFns *bf = nullptr;
-    dolinc_status st = batch_prepare(bt, s, dt, u, ws, ws_bytes, L, &bf);
+    int grid = 0;
+    dolinc_status st = batch_prepare(bt, s, dt, u, ws, ws_bytes, L, &bf, grid);
     if (st) return st;
     cudaStream_t cs = reinterpret_cast<cudaStream_t>(stream);
-    if (!use_graph) return batch_launch_step(bt, s, bf, dt, u, ws, L, cs);
+    if (!use_graph) return batch_launch_step(bt, s, bf, dt, u, ws, L, grid, cs);
     std::ostringstream k;
     k << (const void *)u << '|' << ws << '|' << (const void *)dt << '|' << scheme_key(bt->arena, s) << '|' << s->k << ','
       << s->r << ',' << s->flux << ',' << s->gamma << ',' << s->adv[0] << ',' << s->adv[1] << ',' << s->adv[2] << '|'
-      << bt->block << ',' << bt->grid << ',' << bt->spin_limit;
+      << bt->block << ',' << grid << ',' << bt->spin_limit;
     if (!bt->exec || bt->gkey != k.str()) {
         if (bt->exec) {
             cudaGraphExecDestroy(bt->exec);
@@ -1525,7 +1531,7 @@ dolinc_status dolinc_batch_rk_step(dolinc_batch *bt, const dolinc_scheme *s, con
         if (!bt->cap) CU(cudaStreamCreateWithFlags(&bt->cap, cudaStreamNonBlocking));
         cudaGraph_t g = nullptr;
         CU(cudaStreamBeginCapture(bt->cap, cudaStreamCaptureModeThreadLocal));
-        dolinc_status ls = batch_launch_step(bt, s, bf, dt, u, ws, L, bt->cap);
+        dolinc_status ls = batch_launch_step(bt, s, bf, dt, u, ws, L, grid, bt->cap);
         cudaError_t e = cudaStreamEndCapture(bt->cap, &g);
         cudaGetLastError();
         if (ls) {
@@ -1573,17 +1579,18 @@ dolinc_status dolinc_batch_autotune(dolinc_batch *bt, const dolinc_scheme *s, co
             bt->grid = 0;
             WsLayout L;
             const BatchFns *bf = nullptr;
-            dolinc_status st = batch_prepare(bt, s, dt, u, ws, ws_bytes, L, &bf);
+            int grid = 0;
+            dolinc_status st = batch_prepare(bt, s, dt, u, ws, ws_bytes, L, &bf, grid);
             if (st) continue;
-            bt->grid = std::max(1, (int)(bt->grid * fracs[fi]));
-            if (batch_launch_step(bt, s, bf, dt, u, ws, L, cs)) continue;
+            grid = std::max(1, (int)(grid * fracs[fi]));
+            if (batch_launch_step(bt, s, bf, dt, u, ws, L, grid, cs)) continue;
             cudaEventRecord(e0, cs);
-            for (int r = 0; r < 3; ++r) batch_launch_step(bt, s, bf, dt, u, ws, L, cs);
+            for (int r = 0; r < 3; ++r) batch_launch_step(bt, s, bf, dt, u, ws, L, grid, cs);
             cudaEventRecord(e1, cs);
             cudaEventSynchronize(e1);
             float ms = 0;
             cudaEventElapsedTime(&ms, e0, e1);
-            if (ms / 3 < best) best = ms / 3, best_b = bt->block, best_g = bt->grid;
+            if (ms / 3 < best) best = ms / 3, best_b = bt->block, best_g = grid;
         }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
