@@ -11,6 +11,7 @@
 #include <mutex>
 #include <sstream>
 #include <string>
+#include <tuple>
 #include <vector>
 
 #include "../../include/dolinc.h"
@@ -54,7 +55,9 @@ void init_paths()
     std::memset(g_ind, 0, sizeof g_ind);
     std::memset(g_batch, 0, sizeof g_batch);
     register_indicator(g_ind);
-    register_batch(g_batch);
+    register_batch_f64(g_batch);
+    register_batch_f32(g_batch);
+    register_batch_bf16(g_batch);
     register_paths_d2s_f64(g_paths);
     register_paths_d2s_f32(g_paths);
     register_paths_d2s_bf16(g_paths);
@@ -153,7 +156,7 @@ struct dolinc_batch {
     std::vector<int64_t> cell_off;
     const int32_t *cell_mesh = nullptr;
     int block = 256, grid = 0;         // persistent launch shape (grid 0: as many blocks as fit)
-    std::map<std::pair<const void *, int>, int> fit;   // resident blocks of each kernel and block size
+    std::map<std::tuple<const void *, int, int>, int> fit;   // resident blocks by path, mode and block size
     unsigned spin_limit = 1u << 23;    // polls a grid-barrier wait makes before giving up
     cudaGraphExec_t exec = nullptr;
     cudaStream_t cap = nullptr;        // private stream the graph is captured on
@@ -1445,7 +1448,7 @@ dolinc_status dolinc_batch_workspace_size(const dolinc_batch *b, const dolinc_sc
 
 namespace {
 dolinc_status batch_launch_step(dolinc_batch *bt, const dolinc_scheme *s, const BatchFns *bf, const double *dt,
-                                double *u, void *ws, const WsLayout &L, int grid, cudaStream_t cs)
+                                double *u, void *ws, const WsLayout &L, int mode, int grid, cudaStream_t cs)
 {
     static const double A[3] = {0.0, 0.75, 1.0 / 3.0}, Bc[3] = {1.0, 0.25, 2.0 / 3.0};
     dolinc_mesh *m = bt->arena;
@@ -1470,15 +1473,20 @@ dolinc_status batch_launch_step(dolinc_batch *bt, const dolinc_scheme *s, const 
         static_assert(256 + 4 * BAR_WORDS <= 1024, "barrier words within the cleared head of the workspace");
         b.bar = reinterpret_cast<unsigned *>(B(ws, L.status + 256));
         b.spin_limit = bt->spin_limit;
-        cudaError_t e = bf->launch(m->d, a, b, grid, bt->block, cs);
+        cudaError_t e = bf->launch(m->d, a, b, mode, grid, bt->block, cs);
         if (e != cudaSuccess) return fail(DOLINC_ERR_CUDA, std::string("cooperative launch: ") + cudaGetErrorString(e));
         cur = 1 - cur;
     }
     return DOLINC_OK;
 }
 
+// BATCH_LAT up to this many cells per thread of its own grid.  FP32 at 1.05 turns (40,960
+// tetrahedra, Euler order 5) 145 us a step, BATCH_THR 123; at 0.93 turns (36,200 triangles,
+// Euler order 3) 35 against 53.
+constexpr int64_t kBatchLatTurns = 1;
+
 dolinc_status batch_prepare(dolinc_batch *bt, const dolinc_scheme *s, const double *dt, double *u, void *ws,
-                            size_t ws_bytes, WsLayout &L, const BatchFns **bf, int &grid)
+                            size_t ws_bytes, WsLayout &L, const BatchFns **bf, int &mode, int &grid)
 {
     dolinc_mesh *m = bt->arena;
     dolinc_status st = check_scheme(m, s);
@@ -1493,15 +1501,19 @@ dolinc_status batch_prepare(dolinc_batch *bt, const dolinc_scheme *s, const doub
     if (!(*bf)->launch) return fail(DOLINC_ERR_UNSUPPORTED, "no batched kernel for this scheme");
     // the kernels of a batch's schemes need different registers: each launch takes what fits
     // of its own kernel, an autotuned shape at most its grid
-    int &fit = bt->fit[{*bf, bt->block}];
-    if (fit <= 0) {
+    auto fit = [&](int mode) -> int {
+        int &f = bt->fit[{*bf, mode, bt->block}];
         int sms = 0;
-        CU(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, m->device));
-        const int per = (*bf)->blocks_per_sm(bt->block);
-        if (per <= 0) return fail(DOLINC_ERR_UNSUPPORTED, "batched kernel does not fit on an SM");
-        fit = per * sms;
-    }
-    grid = bt->grid > 0 ? std::min(bt->grid, fit) : fit;
+        if (f <= 0 && cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, m->device) == cudaSuccess)
+            f = (*bf)->blocks_per_sm(mode, bt->block) * sms;
+        return f;
+    };
+    mode = BATCH_LAT;
+    if (s->precision != DOLINC_FP64 && m->h.n_cells > kBatchLatTurns * fit(BATCH_LAT) * bt->block)
+        mode = s->nv == 1 && s->n_diff == ns + 1 ? BATCH_NEXT : BATCH_THR;
+    const int most = fit(mode);
+    if (most <= 0) return fail(DOLINC_ERR_UNSUPPORTED, "batched kernel does not fit on an SM");
+    grid = bt->grid > 0 ? std::min(bt->grid, most) : most;
     return DOLINC_OK;
 }
 }  // namespace
@@ -1512,11 +1524,11 @@ dolinc_status dolinc_batch_rk_step(dolinc_batch *bt, const dolinc_scheme *s, con
     if (!bt) return fail(DOLINC_ERR_INVALID_ARG, "null batch");
     WsLayout L;
     const BatchFns *bf = nullptr;
-    int grid = 0;
-    dolinc_status st = batch_prepare(bt, s, dt, u, ws, ws_bytes, L, &bf, grid);
+    int mode = 0, grid = 0;
+    dolinc_status st = batch_prepare(bt, s, dt, u, ws, ws_bytes, L, &bf, mode, grid);
     if (st) return st;
     cudaStream_t cs = reinterpret_cast<cudaStream_t>(stream);
-    if (!use_graph) return batch_launch_step(bt, s, bf, dt, u, ws, L, grid, cs);
+    if (!use_graph) return batch_launch_step(bt, s, bf, dt, u, ws, L, mode, grid, cs);
     std::ostringstream k;
     k << (const void *)u << '|' << ws << '|' << (const void *)dt << '|' << scheme_key(bt->arena, s) << '|' << s->k << ','
       << s->r << ',' << s->flux << ',' << s->gamma << ',' << s->adv[0] << ',' << s->adv[1] << ',' << s->adv[2] << '|'
@@ -1531,7 +1543,7 @@ dolinc_status dolinc_batch_rk_step(dolinc_batch *bt, const dolinc_scheme *s, con
         if (!bt->cap) CU(cudaStreamCreateWithFlags(&bt->cap, cudaStreamNonBlocking));
         cudaGraph_t g = nullptr;
         CU(cudaStreamBeginCapture(bt->cap, cudaStreamCaptureModeThreadLocal));
-        dolinc_status ls = batch_launch_step(bt, s, bf, dt, u, ws, L, grid, bt->cap);
+        dolinc_status ls = batch_launch_step(bt, s, bf, dt, u, ws, L, mode, grid, bt->cap);
         cudaError_t e = cudaStreamEndCapture(bt->cap, &g);
         cudaGetLastError();
         if (ls) {
@@ -1579,13 +1591,13 @@ dolinc_status dolinc_batch_autotune(dolinc_batch *bt, const dolinc_scheme *s, co
             bt->grid = 0;
             WsLayout L;
             const BatchFns *bf = nullptr;
-            int grid = 0;
-            dolinc_status st = batch_prepare(bt, s, dt, u, ws, ws_bytes, L, &bf, grid);
+            int mode = 0, grid = 0;
+            dolinc_status st = batch_prepare(bt, s, dt, u, ws, ws_bytes, L, &bf, mode, grid);
             if (st) continue;
             grid = std::max(1, (int)(grid * fracs[fi]));
-            if (batch_launch_step(bt, s, bf, dt, u, ws, L, grid, cs)) continue;
+            if (batch_launch_step(bt, s, bf, dt, u, ws, L, mode, grid, cs)) continue;
             cudaEventRecord(e0, cs);
-            for (int r = 0; r < 3; ++r) batch_launch_step(bt, s, bf, dt, u, ws, L, grid, cs);
+            for (int r = 0; r < 3; ++r) batch_launch_step(bt, s, bf, dt, u, ws, L, mode, grid, cs);
             cudaEventRecord(e1, cs);
             cudaEventSynchronize(e1);
             float ms = 0;

@@ -22,6 +22,8 @@
 #include "device_mesh.hpp"
 #include "tma.cuh"
 
+#include <type_traits>
+
 namespace dol {
 
 enum { PREC_F64 = 0, PREC_F32 = 1, PREC_BF16 = 2 };
@@ -929,10 +931,11 @@ __device__ __forceinline__ bool nonfinite64(double x)
     return ((unsigned long long)__double_as_longlong(x) & 0x7ff0000000000000ull) == 0x7ff0000000000000ull;
 }
 
-template <class R>
+// INT: conversions by integer operations (see narrow)
+template <bool INT = true, class R>
 __device__ __forceinline__ double stage_update(const StageArgs &a, long long i, R dtR)
 {
-    const double t = a.us[i] + widen(dtR);
+    const double t = a.us[i] + (INT ? widen(dtR) : (double)dtR);
     // stage 0 (A = 0, B = 1) is t itself; the test on the bits keeps the FP64 pipe free
     return __double_as_longlong(a.A) == 0 ? t : fma(a.B, t, a.A * a.u0[i]);
 }
@@ -1464,7 +1467,7 @@ __device__ __forceinline__ void grid_leave(unsigned *bar, bool clear_abort)
     }
 }
 
-template <int DIM, int NV, int M, int PREC>
+template <int DIM, int NV, int M, int PREC, int UB = diff_batch(NV * ncoef(DIM, M - 1))>
 __device__ __forceinline__ void diff_cell(const DevMesh &mesh, const void *in_v, void *out_v, int c)
 {
     using R = typename PrecT<PREC>::R;
@@ -1483,7 +1486,6 @@ __device__ __forceinline__ void diff_cell(const DevMesh &mesh, const void *in_v,
     poly_mul_acc<DIM, NV, M, R>(acc, x, wx, wy, wz);
     int s0, s1;
     slot_range(mesh, c, s0, s1);
-    constexpr int UB = diff_batch(NV * CI);       // slots whose gathers are in flight together
     for (int s = s0; s < s1; s += UB) {
         R kx[UB], ky[UB], kz[UB], xs[UB][NV * CI];
         int nb[UB];
@@ -1515,8 +1517,28 @@ template <int DIM, int NV, int PREC> struct CoherentSrc {
     __device__ __forceinline__ const R *face(int f) const { return Geo<R>::face(mesh) + 8ll * f; }
 };
 
-template <int DIM, int NV, int NS, int PREC>
-__global__ void __launch_bounds__(256, (NV == 1 && NS == 1 && PREC != PREC_F64) ? 4 : 1) k_batch_stage(DevMesh mesh, StageArgs a, BatchArgs b)
+// Three kernels below FP64 (BatchPath::launch; the host's rule: kBatchLatTurns):
+//   BATCH_LAT   at most one cell per thread of its own grid: registers as needed (one to
+//               three blocks per SM), four gathers and two slots in flight, and the order
+//               above the stencil's, which the stage does not read, in the stage's loop
+//               (n_diff = NS + 1: no barrier between).
+//   BATCH_THR   more cells: occupancy instead.  Registers as the compiler takes them by
+//               itself (a stated minimum of one block lets it take all of them), Euler one
+//               gather at a time, every order before the stage.
+//   BATCH_NEXT  more cells, scalar, n_diff = NS + 1: as BATCH_LAT's loop, four blocks per SM
+//               for order 3.
+// FP64, bound by its arithmetic, always takes BATCH_LAT.  FP32 order 3, us a step: Euler
+// with n_diff 1, LAT / THR, 17k tetrahedra 43 / 57, 123k 115 / 98, 790k triangles 591 / 262;
+// scalar with n_diff 2, LAT / NEXT, 10k triangles 29 / 37, 113k 41 / 37, 400k 88 / 70.
+enum { BATCH_LAT, BATCH_THR, BATCH_NEXT };
+template <int NV, int NS, int MODE> DOL_HD constexpr int batch_min_blocks()
+{
+    return MODE == BATCH_LAT ? 1 : (MODE == BATCH_NEXT && NS == 1) ? 4 : 0;
+}
+
+template <int DIM, int NV, int NS, int PREC, int MODE>
+__global__ void __launch_bounds__(256, batch_min_blocks<NV, NS, MODE>())
+    k_batch_stage(DevMesh mesh, StageArgs a, BatchArgs b)
 {
     using R = typename PrecT<PREC>::R;
     using T0 = typename PrecT<PREC>::T0;
@@ -1524,9 +1546,24 @@ __global__ void __launch_bounds__(256, (NV == 1 && NS == 1 && PREC != PREC_F64) 
     const int tid = blockIdx.x * blockDim.x + threadIdx.x;
     const int n = mesh.n_cells;
     constexpr int S0 = ord_stride<DIM, NV, 0, PREC>();
+    static_assert(MODE != BATCH_NEXT || NV == 1, "scalar schemes");
+    const bool beside = MODE == BATCH_NEXT || (MODE == BATCH_LAT && b.n_diff == NS + 1);
+    // Euler's 4 or 5 conversions a cell hide behind its gathers, so they take the instruction:
+    // 245 -> 234 us a step on 320k tetrahedra, n_diff = 1
+    constexpr bool INT = NV == 1 || MODE == BATCH_LAT;
     unsigned round = 0;
     bool ok = !grid_aborted(b.bar);
     auto sync = [&] { ok = ok && grid_sync(b.bar, ++round, a.status, b.spin_limit); };
+    auto diff = [&](int c, auto order) {
+        constexpr int M = decltype(order)::value;
+        // Euler with many cells: one slot's gather at a time, for the registers
+        constexpr int UB = (NV > 1 && MODE != BATCH_LAT) ? 1 : diff_batch(NV * ncoef(DIM, M - 1));
+        diff_cell<DIM, NV, M, PREC, UB>(mesh, b.ord[M - 1], b.ord[M], c);
+    };
+    auto pass = [&](auto order) {
+        if (ok)
+            for (int c = tid; c < n; c += nthr) diff(c, order);
+    };
     if (ok && b.pack_src) {
         for (int c = tid; c < n; c += nthr) {
             R v[NV];
@@ -1537,50 +1574,46 @@ __global__ void __launch_bounds__(256, (NV == 1 && NS == 1 && PREC != PREC_F64) 
         sync();
     }
     // orders the stage reads, a barrier after each
-    if (ok) {
-        for (int c = tid; c < n; c += nthr) diff_cell<DIM, NV, 1, PREC>(mesh, b.ord[0], b.ord[1], c);
+    pass(std::integral_constant<int, 1>{});
+    sync();
+    if constexpr (NS >= 2) {
+        pass(std::integral_constant<int, 2>{});
         sync();
     }
-    if constexpr (NS >= 2)
-        if (ok) {
-            for (int c = tid; c < n; c += nthr) diff_cell<DIM, NV, 2, PREC>(mesh, b.ord[1], b.ord[2], c);
-            sync();
-        }
-    // Two or three orders above the stencil's: before the stage, so that every barrier comes
-    // before the first write of the output (one such order runs beside the stage)
-    if (NS + 2 <= b.n_diff) {
-        if (ok) {
-            for (int c = tid; c < n; c += nthr) diff_cell<DIM, NV, NS + 1, PREC>(mesh, b.ord[NS], b.ord[NS + 1], c);
-            sync();
-        }
-        if (ok)
-            for (int c = tid; c < n; c += nthr) diff_cell<DIM, NV, NS + 2, PREC>(mesh, b.ord[NS + 1], b.ord[NS + 2], c);
-        if constexpr (NS + 3 <= MAXN)
-            if (NS + 3 <= b.n_diff) {
+    // Orders above the stencil's, but for the one beside the stage: before it, so that every
+    // barrier comes before the first write of the output
+    if constexpr (MODE != BATCH_NEXT)
+        if (!beside && NS + 1 <= b.n_diff) {
+            pass(std::integral_constant<int, NS + 1>{});
+            if (NS + 2 <= b.n_diff) {
                 sync();
-                if (ok)
-                    for (int c = tid; c < n; c += nthr)
-                        diff_cell<DIM, NV, NS + 3, PREC>(mesh, b.ord[NS + 2], b.ord[NS + 3], c);
+                pass(std::integral_constant<int, NS + 2>{});
             }
-    }
-    const bool beside = b.n_diff == NS + 1;
+            if constexpr (NS + 3 <= MAXN)
+                if (NS + 3 <= b.n_diff) {
+                    sync();
+                    pass(std::integral_constant<int, NS + 3>{});
+                }
+        }
     if (!ok) {                            // a barrier gave up: leave the output untouched
         grid_leave(b.bar, false);
         return;
     }
     CoherentSrc<DIM, NV, PREC> src{a, mesh};
     T0 *nxt = static_cast<T0 *>(a.o0_next);
-    auto finish = [&](int c, const R *res, R dtr) {
+    auto step_of = [&](int c) { return narrow<R>(b.dt_tab[__ldg(b.cell_mesh + c)]); };
+    auto finish = [&](int c, const R *res, auto dt_of) {
         R iv, d0, d1, d2;
         ld4<R>(Geo<R>::cellk(mesh) + 4ll * c, d0, d1, d2, iv);
+        const R dtr = dt_of(c);
         bool bad = false;
         R o32[NV];
 #pragma unroll
         for (int v = 0; v < NV; ++v) {
             const R r = res[v] * iv;
-            const double o = stage_update(a, (long long)v * n + c, r * dtr);
+            const double o = stage_update<INT>(a, (long long)v * n + c, r * dtr);
             a.out[(long long)v * n + c] = o;
-            o32[v] = narrow<R>(o);
+            o32[v] = INT ? narrow<R>(o) : (R)o;
             bad |= nonfinite64(o);
         }
         if (nxt) store_rec<T0, NV, S0, R>(nxt, c, o32);
@@ -1594,7 +1627,7 @@ __global__ void __launch_bounds__(256, (NV == 1 && NS == 1 && PREC != PREC_F64) 
         const int work = nf + (beside ? n : 0);
         for (int i = tid; i < work; i += nthr) {
             if (i >= nf) {
-                diff_cell<DIM, NV, NS + 1, PREC>(mesh, b.ord[NS], b.ord[NS + 1], i - nf);
+                diff(i - nf, std::integral_constant<int, NS + 1>{});
                 continue;
             }
             const int P = __ldg(mesh.fo + i), N = __ldg(mesh.fn + i);
@@ -1623,27 +1656,33 @@ __global__ void __launch_bounds__(256, (NV == 1 && NS == 1 && PREC != PREC_F64) 
                     res[v] += (word & 1) ? F : -F;
                 }
             }
-            finish(c, res, narrow<R>(b.dt_tab[__ldg(b.cell_mesh + c)]));
+            finish(c, res, step_of);
         }
     } else {
         // one pass over the cells (face-centric: 190 us a step on 600k triangles against 178)
         for (int c = tid; c < n; c += nthr) {
-            if (beside) diff_cell<DIM, NV, NS + 1, PREC>(mesh, b.ord[NS], b.ord[NS + 1], c);
+            if (beside) diff(c, std::integral_constant<int, NS + 1>{});
             R res[NV];
 #pragma unroll
             for (int v = 0; v < NV; ++v) res[v] = (R)0;
             int s0, s1;
             slot_range(mesh, c, s0, s1);
-            const R dtr = narrow<R>(b.dt_tab[__ldg(b.cell_mesh + c)]);
             const bool own_flag = a.flags && a.flags[c];
-#pragma unroll 2
-            for (int s = s0; s < s1; ++s) {
+            auto add = [&](int s) {
                 R F[NV];
                 slot_flux<DIM, NV, NS, PREC>(mesh, a, src, c, s, own_flag, F);
 #pragma unroll
                 for (int v = 0; v < NV; ++v) res[v] += F[v];
+            };
+            if constexpr (MODE != BATCH_THR) {
+                const R dtr = step_of(c);
+#pragma unroll 2
+                for (int s = s0; s < s1; ++s) add(s);
+                finish(c, res, [&](int) { return dtr; });
+            } else {
+                for (int s = s0; s < s1; ++s) add(s);
+                finish(c, res, step_of);
             }
-            finish(c, res, dtr);
         }
     }
     grid_leave(b.bar, false);

@@ -331,12 +331,24 @@ template <int DIM, int NV, int NS, int PREC> struct Path {
 
 // Persistent batched stage (k_batch_stage), launched cooperatively.
 struct BatchFns {
-    cudaError_t (*launch)(const DevMesh &, const StageArgs &, const BatchArgs &, int grid, int block, cudaStream_t);
-    int (*blocks_per_sm)(int block);
+    // mode: BATCH_* (FP64 has BATCH_LAT alone, Euler no BATCH_NEXT)
+    cudaError_t (*launch)(const DevMesh &, const StageArgs &, const BatchArgs &, int mode, int grid, int block,
+                          cudaStream_t);
+    int (*blocks_per_sm)(int mode, int block);
 };
 
 template <int DIM, int NV, int NS, int PREC> struct BatchPath {
-    static cudaError_t launch(const DevMesh &m, const StageArgs &a, const BatchArgs &b, int grid, int block,
+    using Kern = void (*)(DevMesh, StageArgs, BatchArgs);
+    static Kern kernel(int mode)
+    {
+        if constexpr (PREC != PREC_F64) {
+            if constexpr (NV == 1)
+                if (mode == BATCH_NEXT) return k_batch_stage<DIM, NV, NS, PREC, BATCH_NEXT>;
+            if (mode != BATCH_LAT) return k_batch_stage<DIM, NV, NS, PREC, BATCH_THR>;
+        }
+        return k_batch_stage<DIM, NV, NS, PREC, BATCH_LAT>;
+    }
+    static cudaError_t launch(const DevMesh &m, const StageArgs &a, const BatchArgs &b, int mode, int grid, int block,
                               cudaStream_t s)
     {
         cudaLaunchConfig_t cfg = {};
@@ -348,12 +360,12 @@ template <int DIM, int NV, int NS, int PREC> struct BatchPath {
         attr[0].val.cooperative = 1;
         cfg.attrs = attr;
         cfg.numAttrs = 1;
-        return cudaLaunchKernelEx(&cfg, k_batch_stage<DIM, NV, NS, PREC>, m, a, b);
+        return cudaLaunchKernelEx(&cfg, kernel(mode), m, a, b);
     }
-    static int blocks_per_sm(int block)
+    static int blocks_per_sm(int mode, int block)
     {
         int n = 0;
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_batch_stage<DIM, NV, NS, PREC>, block, 0);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel(mode), block, 0);
         return n;
     }
     static BatchFns fns() { return BatchFns{&launch, &blocks_per_sm}; }
@@ -362,7 +374,23 @@ template <int DIM, int NV, int NS, int PREC> struct BatchPath {
 // batch table index: dim (2,3) x nv-class x NS (1, 2) x precision
 inline int batch_index(int dim, int nv, int ns, int prec) { return (((dim - 2) * 2 + (nv == 1 ? 0 : 1)) * 2 + (ns - 1)) * 3 + prec; }
 constexpr int N_BATCH = 2 * 2 * 2 * 3;
-void register_batch(BatchFns *t);
+// one translation unit per precision (compiled in parallel)
+template <int PREC> inline void register_batch(BatchFns *t)
+{
+    auto reg = [&](auto dim, auto nv) {
+        constexpr int D = decltype(dim)::value, V = decltype(nv)::value;
+        t[batch_index(D, V, 1, PREC)] = BatchPath<D, V, 1, PREC>::fns();
+        t[batch_index(D, V, 2, PREC)] = BatchPath<D, V, 2, PREC>::fns();
+    };
+    using std::integral_constant;
+    reg(integral_constant<int, 2>{}, integral_constant<int, 1>{});
+    reg(integral_constant<int, 2>{}, integral_constant<int, 4>{});
+    reg(integral_constant<int, 3>{}, integral_constant<int, 1>{});
+    reg(integral_constant<int, 3>{}, integral_constant<int, 5>{});
+}
+void register_batch_f64(BatchFns *t);
+void register_batch_f32(BatchFns *t);
+void register_batch_bf16(BatchFns *t);
 
 // table index: dim (2,3) x nv-class (scalar, Euler) x NS (1..4) x precision (3)
 inline int path_index(int dim, int nv, int ns, int prec)
