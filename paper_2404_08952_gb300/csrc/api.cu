@@ -1,6 +1,7 @@
 // C ABI of the DOLINC stage library (include/dolinc.h).
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -103,6 +104,18 @@ struct dolinc_mesh {
     int bv_nv = 0;                     // variables of the boundary values set (0: none yet)
     std::vector<int32_t> bidx_h;       // host copy of DevMesh::bidx
     int max_faces = 0;                 // largest number of slots of a cell
+    // of the whole mesh (a part: the mesh it was cut from), whose FP64 shape, and so bits, a
+    // part takes: its cells, its largest number of slots, has it Dirichlet or Neumann faces
+    int64_t whole_cells = 0;
+    int whole_faces = 0;
+    bool whole_bc = false;
+    void set_whole(const HostMesh &g)
+    {
+        whole_cells = g.n_cells;
+        whole_faces = 0;
+        for (int64_t c = 0; c < g.n_cells; ++c) whole_faces = std::max(whole_faces, (int)(g.off[c + 1] - g.off[c]));
+        whole_bc = std::any_of(g.fkind.begin(), g.fkind.end(), [](int8_t k) { return k >= 2; });
+    }
     unsigned *steps_bar = nullptr;     // BAR_WORDS grid-barrier words of k_steps_small, zero between launches
     unsigned steps_spin = 1u << 22;    // polls one of its barrier waits makes before giving up
     std::map<std::string, Tune> tuned;  // launch shapes chosen by dolinc_autotune, per scheme
@@ -372,7 +385,22 @@ std::string scheme_key(const dolinc_mesh *m, const dolinc_scheme *s)
 // no slower than one lane per slot: a step on 20k tetrahedra takes 59 us against 46, on
 // 40k 69 against 67, on 69k 73 against 80; 33k / 65k triangles 55 / 60 us against 49 / 65.
 constexpr int64_t kTreeCells = 40000;
+// FP64 up to this many cells: one lane per slot.  A call there is its launches and the
+// longest chain of loads and FP64 operations, and lanes take one launch less and a quarter
+// of the chain.  Residual, lanes / slot order, us: 2k triangles 20.5 / 22.8 (Euler 26 / 32),
+// 2.6k tetrahedra 21.6 / 24.7 (35.8 / 40.1), 2.6k hexes and prisms 24.7 / 29.6 (44 / 47); 8k
+// triangles 21.8 / 24.4 (34.9 / 32.9), 8.6k tetrahedra 24.6 / 26.7 (44 / 41), 20k triangles
+// 30.8 / 24.7 (67 / 38).  Order-5 step, 2.6k tetrahedra 91 / 101 (Euler 216 / 234), 20k 282 /
+// 199; steps that read order 1 alone are no slower in slot order from 2k cells (n_diff 3, 2k
+// triangles Euler 80 / 72), but with Dirichlet faces 54 / 60 at 2k.
+constexpr int64_t kLaneCells64 = 4000;
 
+bool is_tuned(const dolinc_mesh *m, const dolinc_scheme *s)
+{
+    return !m->tuned.empty() && m->tuned.count(scheme_key(m, s));
+}
+
+// Launch shape of the step entry points.
 Tune tune_for(const dolinc_mesh *m, const dolinc_scheme *s)
 {
     if (!m->tuned.empty()) {
@@ -380,9 +408,11 @@ Tune tune_for(const dolinc_mesh *m, const dolinc_scheme *s)
         if (it != m->tuned.end()) return it->second;
     }
     Tune t;
-    const int lanes = m->max_faces <= 4 ? 4 : 8;
+    const int lanes = (s->precision == DOLINC_FP64 ? m->whole_faces : m->max_faces) <= 4 ? 4 : 8;
     t.diff_lpc = t.stage_lpc = lanes;             // one lane per face slot
     if (s->precision == DOLINC_FP64) {
+        // The schemes that k_steps_small takes keep its slot order on every path.
+        if (m->whole_cells <= kLaneCells64 && (needed_order(*s) >= 2 || m->whole_bc)) return t;
         // slot order; unpaired passes (the second runs beside the stage): a step on 69k
         // tetrahedra takes 352 us, paired 383, one lane per slot 662
         t.diff_lpc = 1;
@@ -401,6 +431,17 @@ Tune tune_for(const dolinc_mesh *m, const dolinc_scheme *s)
         }
     }
     return t;
+}
+
+// Launch shape of one residual or stage evaluation.
+Tune tune_eval(const dolinc_mesh *m, const dolinc_scheme *s)
+{
+    if (s->precision == DOLINC_FP64 && m->whole_cells <= kLaneCells64 && !is_tuned(m, s)) {
+        Tune t;
+        t.diff_lpc = t.stage_lpc = m->whole_faces <= 4 ? 4 : 8;
+        return t;
+    }
+    return tune_for(m, s);
 }
 
 // differential passes 1..n from the order-0 record at o0off
@@ -553,6 +594,7 @@ dolinc_status upload_mesh(dolinc_mesh *m)
     std::vector<int32_t> off(h.off.begin(), h.off.end());
     m->max_faces = 0;
     for (int64_t c = 0; c < nc; ++c) m->max_faces = std::max(m->max_faces, (int)(h.off[c + 1] - h.off[c]));
+    m->set_whole(h);
     // first internal face owned by each cell (faces are sorted by owner)
     std::vector<int32_t> fown(nc + 1, 0);
     for (int64_t f = 0; f < nf; ++f) fown[h.fo[f] + 1]++;
@@ -767,11 +809,12 @@ dolinc_status dolinc_residual(dolinc_mesh *m, const dolinc_scheme *s, const doub
     if (!p) return fail(DOLINC_ERR_UNSUPPORTED, "no kernel for this (dim, nv, order, precision)");
     cudaStream_t cs = reinterpret_cast<cudaStream_t>(stream);
     timed(m, DOLINC_KERNEL_PACK, cs, [&] { p->pack(m->d, u, B(ws, L.o0[0]), nullptr, cs); });
-    run_diffs(m, p, ws, L, L.o0[0], s->n_diff, tune_for(m, s), cs);
+    const Tune tn = tune_eval(m, s);
+    run_diffs(m, p, ws, L, L.o0[0], s->n_diff, tn, cs);
     StageArgs a = base_args(m, s, ws, L, L.o0[0]);
     a.mode = 0;
     a.out = R;
-    timed(m, DOLINC_KERNEL_STAGE, cs, [&] { p->stage(m->d, a, tune_for(m, s), cs); });
+    timed(m, DOLINC_KERNEL_STAGE, cs, [&] { p->stage(m->d, a, tn, cs); });
     return launch_check();
 }
 
@@ -789,7 +832,8 @@ dolinc_status dolinc_rk_stage(dolinc_mesh *m, const dolinc_scheme *s, double dt,
     if (!p) return fail(DOLINC_ERR_UNSUPPORTED, "no kernel for this (dim, nv, order, precision)");
     cudaStream_t cs = reinterpret_cast<cudaStream_t>(stream);
     timed(m, DOLINC_KERNEL_PACK, cs, [&] { p->pack(m->d, us, B(ws, L.o0[0]), nullptr, cs); });
-    run_diffs(m, p, ws, L, L.o0[0], s->n_diff, tune_for(m, s), cs);
+    const Tune tn = tune_eval(m, s);
+    run_diffs(m, p, ws, L, L.o0[0], s->n_diff, tn, cs);
     StageArgs a = base_args(m, s, ws, L, L.o0[0]);
     a.mode = 1;
     a.u0 = u0;
@@ -799,7 +843,7 @@ dolinc_status dolinc_rk_stage(dolinc_mesh *m, const dolinc_scheme *s, double dt,
     a.B = Bc[stage];
     set_dt(a, dt);
     a.o0_next = nullptr;
-    timed(m, DOLINC_KERNEL_STAGE, cs, [&] { p->stage(m->d, a, tune_for(m, s), cs); });
+    timed(m, DOLINC_KERNEL_STAGE, cs, [&] { p->stage(m->d, a, tn, cs); });
     return launch_check();
 }
 
@@ -820,7 +864,7 @@ bool small_steps_ok(const dolinc_mesh *m, const PathFns *p, const dolinc_scheme 
 {
     return p->steps_small && s->n_diff <= 2 && m->max_faces <= 8 &&
            m->h.n_cells <= (s->precision == DOLINC_FP64 && s->nv > 1 ? kSmallCellsEuler64 : kSmallCells) &&
-           m->d.n_bcell == 0 && !m->prof && !m->part && (m->tuned.empty() || !m->tuned.count(scheme_key(m, s)));
+           m->d.n_bcell == 0 && !m->prof && !m->part && !is_tuned(m, s);
 }
 
 cudaError_t small_steps(dolinc_mesh *m, const PathFns *p, const dolinc_scheme *s, double dt, double *u, void *ws,
@@ -1945,6 +1989,7 @@ dolinc_status dolinc_mesh_create_part(const dolinc_mesh_desc *desc, const int32_
         delete m;
         return st;
     }
+    m->set_whole(g);
     std::vector<int32_t> sc(ps->plan.send_cells.begin(), ps->plan.send_cells.end());
     std::vector<int32_t> rc(ps->plan.recv_cells.begin(), ps->plan.recv_cells.end());
     sc.push_back(0);                            // never empty
