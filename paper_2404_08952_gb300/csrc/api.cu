@@ -382,9 +382,12 @@ std::string scheme_key(const dolinc_mesh *m, const dolinc_scheme *s)
 }
 
 // From this many cells one thread per cell (and the face-centric stage's extra launch) is
-// no slower than one lane per slot: a step on 20k tetrahedra takes 59 us against 46, on
-// 40k 69 against 67, on 69k 73 against 80; 33k / 65k triangles 55 / 60 us against 49 / 65.
-constexpr int64_t kTreeCells = 40000;
+// as fast as one lane per slot.  Four slots, order 3, n_diff 2 (few passes), lanes / one
+// thread, us: residual on 40k triangles 18.5 / 20.5, 44k tetrahedra 18.7 / 20.5 (Euler 27.4 /
+// 28.1), 54k triangles Euler 23.7 / 20.5, 58k tetrahedra 24.4 / 21.2; step on 44k tetrahedra
+// Euler 59.4 / 61.2, 58k 67.3 / 63.2.  More passes or eight slots, step: 40k triangles n_diff 3
+// 51.7 / 48.0, 40k tetrahedra order 5 89 / 75, 40k hexes and prisms 57.7 / 46.9.
+constexpr int64_t kTreeCells = 40000, kTreeCellsFew = 50000;
 // FP64 up to this many cells: one lane per slot.  A call there is its launches and the
 // longest chain of loads and FP64 operations, and lanes take one launch less and a quarter
 // of the chain.  Residual, lanes / slot order, us: 2k triangles 20.5 / 22.8 (Euler 26 / 32),
@@ -419,7 +422,8 @@ Tune tune_for(const dolinc_mesh *m, const dolinc_scheme *s)
         t.diff_block = 64;
         t.stage_lpc = -2;
         t.stage_block = 64;
-    } else if (m->max_faces <= lanes && m->h.n_cells >= kTreeCells) {
+    } else if (m->max_faces <= lanes &&
+               m->h.n_cells >= (lanes == 4 && s->n_diff <= 2 && needed_order(*s) == 1 ? kTreeCellsFew : kTreeCells)) {
         t.diff_lpc = 1;
         t.diff_block = 64;
         t.tree = lanes;

@@ -92,3 +92,26 @@ def test_every_path_of_a_step_sums_alike(name, order, n_diff, values):
         dg.dolinc_sync_status(P, w)
         own = P.plan["owned"].astype(bool)
         np.testing.assert_array_equal(x.cpu().numpy()[:, own], whole[:, P.plan["local_cells"][own]])
+
+
+@pytest.mark.parametrize("flux,precision,n_diff", [("upwind", "fp32", 2), ("rusanov", "fp32", 2), ("rusanov", "fp32", 1),
+                                                   ("burgers", "fp32_bf16", 2)])
+@pytest.mark.parametrize("nx", [149, 162])                # 47,680 and 51,840 cells: both sides of the limit
+def test_few_passes_give_the_lane_bits_on_both_sides(flux, precision, n_diff, nx):
+    m = synth.tri_mesh(nx, 160, 0.2, 3)
+    M = dg.Mesh(m)
+    nv = 4 if flux == "rusanov" else 1
+    sch = dg.Scheme(k=3, r=1, n_diff=n_diff, flux=flux, nv=nv, precision=precision, adv=(1.0, 0.7))
+    s = 0.1 * np.random.default_rng(2).random(M.n_cells)
+    u0 = torch.from_numpy((1.0 + s)[None] if nv == 1 else np.stack([1.0 + s, 0.4 + s, 0.2 - s, 3.0 + s])).cuda()
+    out = []
+    for tuned in (False, True):
+        if tuned:
+            dg.dolinc_set_tuning(M, sch, 4, 256, 4, 128)
+        ws = dg.workspace(M, sch)
+        u, R = u0.clone(), torch.empty_like(u0)
+        dg.dolinc_residual(M, sch, u, R, ws)
+        dg.dolinc_rk_steps(M, sch, 1e-4, 2, u, ws)
+        dg.dolinc_sync_status(M, ws)
+        out.append((u, R))
+    assert torch.equal(out[0][0], out[1][0]) and torch.equal(out[0][1], out[1][1])
