@@ -414,8 +414,11 @@ Tune tune_for(const dolinc_mesh *m, const dolinc_scheme *s)
     const int lanes = (s->precision == DOLINC_FP64 ? m->whole_faces : m->max_faces) <= 4 ? 4 : 8;
     t.diff_lpc = t.stage_lpc = lanes;             // one lane per face slot
     if (s->precision == DOLINC_FP64) {
-        // The schemes that k_steps_small takes keep its slot order on every path.
-        if (m->whole_cells <= kLaneCells64 && (needed_order(*s) >= 2 || m->whole_bc)) return t;
+        // The schemes that k_steps_small takes keep its slot order on every path.  Eight lanes
+        // with n_diff 3 or 4: 324 hexes and prisms 66 / 97 us a step, slot order 67 / 115
+        // (Euler 146 / 247 and 158 / 291).
+        if (m->whole_cells <= kLaneCells64 && (needed_order(*s) >= 2 || m->whole_bc || (lanes == 8 && s->n_diff >= 3)))
+            return t;
         // slot order; unpaired passes (the second runs beside the stage): a step on 69k
         // tetrahedra takes 352 us, paired 383, one lane per slot 662
         t.diff_lpc = 1;
@@ -861,13 +864,16 @@ namespace {
 // Measured per step, one launch against separate ones: 4k / 16k / 39k triangles FP32 Euler
 // 25 / 31 / 49 us against 54 / 50 / 54, 40k tetrahedra 65 against 67; FP64 advection on 8k /
 // 39k triangles 44 / 74 us against 58 / 81.  FP64 Euler needs twice the registers, so the
-// one resident grid holds fewer warps: 2.6k / 8.6k / 20k tetrahedra 77 / 107 / 182 us against
-// 92 / 141 / 167, 8k / 16k triangles 79 / 103 against 77 / 98.
-constexpr int64_t kSmallCells = 40000, kSmallCellsEuler64 = 8000;
+// one resident grid holds fewer warps: 2.6k / 8.6k / 11.8k / 13.7k tetrahedra 77 / 104 / 99 /
+// 145 us against 92 / 135 / 139 / 139 (one lane per slot: 117 at 8.6k), 8.7k / 12k hexes and
+// prisms 116 / 162 against 159 / 164, 8k / 16k triangles 79 / 103 against 77 / 98.
+constexpr int64_t kSmallCells = 40000, kSmallCellsEuler64 = 8000, kSmallCellsEuler64_3d = 12500;
 bool small_steps_ok(const dolinc_mesh *m, const PathFns *p, const dolinc_scheme *s)
 {
-    return p->steps_small && s->n_diff <= 2 && m->max_faces <= 8 &&
-           m->h.n_cells <= (s->precision == DOLINC_FP64 && s->nv > 1 ? kSmallCellsEuler64 : kSmallCells) &&
+    const int64_t most = s->precision != DOLINC_FP64 || s->nv == 1 ? kSmallCells
+                         : m->h.dim == 3                           ? kSmallCellsEuler64_3d
+                                                                   : kSmallCellsEuler64;
+    return p->steps_small && s->n_diff <= 2 && m->max_faces <= 8 && m->h.n_cells <= most &&
            m->d.n_bcell == 0 && !m->prof && !m->part && !is_tuned(m, s);
 }
 
