@@ -398,6 +398,23 @@ constexpr int64_t kTreeCells = 40000, kTreeCellsFew = 50000;
 // triangles Euler 80 / 72), but with Dirichlet faces 54 / 60 at 2k.
 constexpr int64_t kLaneCells64 = 4000;
 
+// Bytes of a stage (weights, records of every order, faces and fluxes) from which the tree
+// passes load their weights evict-first.  Below, the next pass or stage finds them in the L2
+// (129 MB).  us a step, evict-first / not: 112 MB (274k tetrahedra Euler) 167 / 165, 117 MB
+// (324k hexes and prisms, order 5) 249 / 226, 140 MB (720k triangles, order 5) 233 / 210,
+// 167 MB (720k triangles Euler) 200 / 200, 203 MB (1.05M triangles, order 5) 320 / 314, 229 MB
+// (633k hexes and prisms, order 5) 457 / 469, 243 MB (1.05M triangles Euler) 277 / 288.
+constexpr size_t kOnceBytes = 215000000;
+
+size_t stage_bytes(const dolinc_mesh *m, const dolinc_scheme *s)
+{
+    const size_t nc = m->h.n_cells, b = elem_bytes(s->precision, 0);
+    size_t n = 4 * b * (m->h.n_slots + nc) + (8 + s->nv) * b * m->h.n_faces;
+    for (int mm = 0; mm <= s->n_diff; ++mm)
+        n += nc * stride_h(m->h.dim, s->nv, mm, s->precision) * elem_bytes(s->precision, mm);
+    return n;
+}
+
 bool is_tuned(const dolinc_mesh *m, const dolinc_scheme *s)
 {
     return !m->tuned.empty() && m->tuned.count(scheme_key(m, s));
@@ -430,6 +447,7 @@ Tune tune_for(const dolinc_mesh *m, const dolinc_scheme *s)
         t.diff_lpc = 1;
         t.diff_block = 64;
         t.tree = lanes;
+        t.once = stage_bytes(m, s) > kOnceBytes;
         // WENO5's weights amplify the rounding of its fused products, which the compiler
         // chooses per kernel: its stage keeps the lane kernel and that kernel's bits
         if (s->limiter != DOLINC_LIMIT_WENO5_ALL && s->limiter != DOLINC_LIMIT_WENO5_FLAGGED) {

@@ -105,18 +105,17 @@ __device__ __forceinline__ void ldg32(const void *p, unsigned *w)
 }
 
 // The same, and 16 bytes, for geometry that a kernel reads once: first to leave the L2,
-// which keeps the records and fluxes that the next kernels read.  Face records in k_flux and
-// weights in k_diff_tree: 630k hexes and prisms order 5 465 -> 452 us a step, 553k
-// tetrahedra order 4 380 -> 374, 1.05M triangles network and step 492 -> 487.  (Not in the
-// paired passes, whose halves share the weights: 2442 -> 2505 us for four steps of 1.31M
-// tetrahedra.)
+// which keeps the records and fluxes that the next kernels read.  Face records in k_flux:
+// 630k hexes and prisms order 5 465 -> 452 us a step, 553k tetrahedra order 4 380 -> 374.
+// Weights in k_diff_tree: where a stage is much larger than the L2 (the host's kOnceBytes).
+// (Not in the paired passes, whose halves share the weights: 2442 -> 2505 us for four steps
+// of 1.31M tetrahedra.)
 __device__ __forceinline__ void ldg32_once(const void *p, unsigned *w)
 {
     asm("ld.global.nc.L2::evict_first.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
         : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]), "=r"(w[4]), "=r"(w[5]), "=r"(w[6]), "=r"(w[7])
         : "l"(p));
 }
-// (first: false where the whole stage fits the L2 and the next stage finds the weights there)
 __device__ __forceinline__ unsigned long long policy_once(bool first)
 {
     unsigned long long p, q;

@@ -325,13 +325,14 @@ __device__ __forceinline__ void diff_cells(const DevMesh &mesh, const void *__re
 // a lane without a slot adding zero.  Cells have at most TREE slots (checked by the
 // launcher).  A pair of lanes is loaded at a time (all of them when the records are
 // small), so that their gathers overlap.
+// evict_first: the weights are first to leave the L2 (the host's rule: kOnceBytes).
 // Why one thread: TREE lanes hold TREE accumulators, exchange them by shuffles and leave
 // lanes idle (5.3 of 8 on hexes and prisms); the pass then waits on issue slots and
 // shuffles instead of on memory.
 template <int DIM, int NV, int M, int PREC, int TREE>
 __device__ __forceinline__ void diff_cells_tree(const DevMesh &mesh, const void *__restrict__ in_v,
                                                 void *__restrict__ out_v, int c, int t, int nt, long long c0,
-                                                unsigned char *smo)
+                                                unsigned char *smo, bool evict_first)
 {
     using R = typename PrecT<PREC>::R;
     using TI = typename OrdT<PREC, M - 1>::T;
@@ -348,9 +349,7 @@ __device__ __forceinline__ void diff_cells_tree(const DevMesh &mesh, const void 
         int s0, s1;
         slot_range(mesh, c, s0, s1);
         const int ns = s1 - s0;
-        // 2^20 slots: a stage of such a mesh moves about 100 MB (181k triangles, 0.5M slots,
-        // criterion and WENO5 step 194 us; evict-first 205)
-        const unsigned long long once = policy_once(mesh.n_slots >= (1 << 20));
+        const unsigned long long once = policy_once(evict_first);
         // slots in the order the tree adds them, two at a time: (0, H), (2, H + 2), (1, ..)
         constexpr int H = TREE / 2, NP = TREE / 2;
         constexpr bool ALL = NV * CI <= 10;          // small records: every gather before the first sum
@@ -446,11 +445,12 @@ __device__ __forceinline__ void diff_cells_tree(const DevMesh &mesh, const void 
 }
 
 template <int DIM, int NV, int M, int PREC, int TREE>
-__global__ void __launch_bounds__(128) k_diff_tree(DevMesh mesh, const void *__restrict__ in_v, void *__restrict__ out_v)
+__global__ void __launch_bounds__(128) k_diff_tree(DevMesh mesh, const void *__restrict__ in_v, void *__restrict__ out_v,
+                                                  bool evict_first)
 {
     extern __shared__ __align__(16) unsigned char smo[];
     diff_cells_tree<DIM, NV, M, PREC, TREE>(mesh, in_v, out_v, (int)(blockIdx.x * blockDim.x + threadIdx.x), threadIdx.x,
-                                            blockDim.x, (long long)blockIdx.x * blockDim.x, smo);
+                                            blockDim.x, (long long)blockIdx.x * blockDim.x, smo, evict_first);
 }
 
 template <int DIM, int NV, int M, int PREC, int LPC>

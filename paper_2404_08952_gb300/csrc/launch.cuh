@@ -16,6 +16,7 @@ struct Tune {
     // (stage_lpc -2) sum in the order of that many lanes per cell (cells of at most
     // `tree` slots, bulk precision below FP64); 0: in slot order
     int tree = 0;
+    bool once = false;           // the tree passes load their weights evict-first
 };
 
 // Grid of a persistent kernel: resident CTAs per SM x SMs (cached per kernel and
@@ -83,13 +84,14 @@ template <int DIM, int NV, int NS, int PREC> struct Path {
         k_diff<DIM, NV, MM, PREC, 1><<<nblk(m.n_cells, bs), bs, out_smem<MM>(bs), s>>>(m, in, out);
     }
     // one thread per cell, summing in the order of TREE lanes
-    template <int TREE> static void diff_tree(const DevMesh &m, int M, const void *in, void *out, cudaStream_t s)
+    template <int TREE>
+    static void diff_tree(const DevMesh &m, int M, const void *in, void *out, bool once, cudaStream_t s)
     {
         constexpr int BS = 64;   // its staged output records stay below 48 KB for every order
         auto go = [&](auto mc) {
             constexpr int MM = decltype(mc)::value;
             static_assert(BS * out_rec_bytes<MM>() <= 48 * 1024, "staged records without an opt-in");
-            k_diff_tree<DIM, NV, MM, PREC, TREE><<<nblk(m.n_cells, BS), BS, out_smem<MM>(BS), s>>>(m, in, out);
+            k_diff_tree<DIM, NV, MM, PREC, TREE><<<nblk(m.n_cells, BS), BS, out_smem<MM>(BS), s>>>(m, in, out, once);
         };
         switch (M) {
         case 1: go(std::integral_constant<int, 1>{}); break;
@@ -215,8 +217,8 @@ template <int DIM, int NV, int NS, int PREC> struct Path {
             return;
         }
         if constexpr (PREC != PREC_F64) {
-            if (t.tree == 4) return diff_tree<4>(m, M, in, out, s);
-            if (t.tree == 8) return diff_tree<8>(m, M, in, out, s);
+            if (t.tree == 4) return diff_tree<4>(m, M, in, out, t.once, s);
+            if (t.tree == 8) return diff_tree<8>(m, M, in, out, t.once, s);
         }
         switch (t.diff_lpc) {
         case 4: diff_l<4>(m, M, in, out, t.diff_block, s); break;
