@@ -213,8 +213,9 @@ dolinc_status dolinc_rk_stage(dolinc_mesh *mesh, const dolinc_scheme *scheme, do
  * the bulk precision; the stage inputs exist only as bulk-precision records and the
  * FP64 state receives one add per step.
  * Untuned steps of a small mesh (up to 40000 cells, stencil order 1, n_diff <= 2) run in
- * one cooperative launch whose grid barriers wait a bounded time: a wait that gives up is
- * reported as DOLINC_ERR_DEVICE_TIMEOUT by dolinc_sync_status and leaves u_dev undefined. */
+ * one cooperative launch whose grid barriers wait a bounded time
+ * (dolinc_mesh_set_spin_limit): a wait that gives up is reported as
+ * DOLINC_ERR_DEVICE_TIMEOUT by dolinc_sync_status and leaves u_dev undefined. */
 dolinc_status dolinc_rk_step(dolinc_mesh *mesh, const dolinc_scheme *scheme, double dt, double *u_dev,
                              void *ws_dev, size_t ws_bytes, dolinc_stream stream);
 
@@ -379,7 +380,8 @@ typedef struct dolinc_batch dolinc_batch;
 dolinc_status dolinc_batch_create(dolinc_mesh *const *meshes, int n, dolinc_batch **out);
 void dolinc_batch_destroy(dolinc_batch *batch);
 dolinc_status dolinc_batch_info(const dolinc_batch *batch, int64_t *n_cells, int64_t *cell_offsets /* [n+1] */);
-/* Polls a grid-barrier wait makes (about 0.1 us each) before it gives up (default 2^23).
+/* Polls a grid-barrier wait makes (one load through the L2 each) before it gives up
+ * (default 2^23).
  * 0 makes every wait give up at once: a way to exercise the timeout path. */
 dolinc_status dolinc_batch_set_spin_limit(dolinc_batch *batch, unsigned polls);
 dolinc_status dolinc_batch_workspace_size(const dolinc_batch *batch, const dolinc_scheme *scheme, size_t *bytes);

@@ -1405,9 +1405,9 @@ __global__ void __launch_bounds__(TILE) k_diff_tile(DevMesh mesh, const void *__
 // flux, residual and update, the phases separated by a grid-wide barrier.  Records
 // written in one phase are read in a later phase of the same launch, so this kernel
 // reads through the coherent path (no read-only loads).  Each barrier waits at most
-// `spin_limit` polls; a wait that gives up sets status bit 1 and an abort word that
-// makes every later barrier, and every later launch until the words are cleared, return at
-// once.
+// `spin_limit` polls; a wait that gives up ends the launch in every block (grid_sync) and
+// sets status bit 1 and an abort word, on which later launches return at once until the
+// words are cleared.
 struct BatchArgs {
     const double *pack_src;      // non-null: phase 0 packs this FP64 field into ord[0]
     void *ord[MAXN + 1];         // order records 0..n_diff
@@ -1701,9 +1701,9 @@ __global__ void __launch_bounds__(256, batch_min_blocks<NV, NS, MODE>())
 //     idle lanes: three times the FP64 instructions on triangles.
 // As separate launches a step of any mesh of up to 16k cells costs 46 us, 4.6 us for each
 // of its ten launches, whatever the size.
-// Each wait polls at most spin_limit times; one that gives up sets status bit 1 and its
-// block leaves (the others' waits then give up too).  The last block to leave clears the
-// barrier words for the next launch.
+// Each wait polls at most spin_limit times; one that gives up ends the launch in every block
+// and sets status bit 1 (grid_sync).  The last block to leave clears the barrier words for
+// the next launch.
 struct StepsArgs {
     StageArgs a;                 // common fields (status, scheme, flags)
     double *u, *ust;             // FP64 state, and the stage value (FP64 path)
