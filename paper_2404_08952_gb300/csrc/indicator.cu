@@ -289,9 +289,17 @@ __global__ void __launch_bounds__(128, 4) k_mlp_infer(const uint2 *__restrict__ 
                                                    DevMesh mesh, const float *__restrict__ own)
 {
     __shared__ uint32_t sx[4][32][XW];
-    __shared__ uint2 sfrag[N_FRAGS * 32];
+    __shared__ __align__(16) uint2 sfrag[N_FRAGS * 32];
     __shared__ float sbias[3 * MLP_H + 1];
-    for (int i = threadIdx.x; i < N_FRAGS * 32; i += blockDim.x) sfrag[i] = frag[i];
+    // all loads of the weights in flight together: a call on 1000 rows 4.6 -> 3.7 us (16 rows per
+    // warp took 3.9), on 1M rows 56.8 -> 55.6
+    static_assert(N_FRAGS * 32 % 2 == 0, "16-byte pieces");
+    constexpr int NW = N_FRAGS * 16;
+#pragma unroll
+    for (int k = 0; k < (NW + 127) / 128; ++k) {
+        const int i = threadIdx.x + 128 * k;
+        if (i < NW) reinterpret_cast<uint4 *>(sfrag)[i] = __ldg(reinterpret_cast<const uint4 *>(frag) + i);
+    }
     for (int i = threadIdx.x; i < MLP_H; i += blockDim.x) {
         sbias[i] = __bfloat162float(__float2bfloat16_rn(theta[OFF_B1 + i]));
         sbias[MLP_H + i] = __bfloat162float(__float2bfloat16_rn(theta[OFF_B2 + i]));
